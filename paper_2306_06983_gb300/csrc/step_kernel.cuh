@@ -948,6 +948,337 @@ __device__ __forceinline__ void mass_flux(const StepParams &P, const float (&gx)
     my = -P.mob * ay;
 }
 
+// Ghost row beyond a wetting wall (Sec. 4.2): its mirror image ph plus
+// (2k - 1) s_p, s_p = phi_p sum_q (4/eps) cos theta_pq phi_q at the image
+// node, so that the difference across the wall is s_p (n_w pointing into the
+// wall); ra < 0 or ra >= ny is the ghost row.
+template <int NS>
+__device__ __forceinline__ void wet_ghost(const StepParams &P, int ra, float (&ph)[NS])
+{
+    const int w = ra < 0 ? 0 : 1;
+    const float k2 = (float)(2 * (ra < 0 ? -ra : ra - (P.ny - 1)) - 1);
+    float phN = 1.f;
+#pragma unroll
+    for (int p = 0; p < NS; ++p) phN -= ph[p];
+    float sp[NS];
+#pragma unroll
+    for (int p = 0; p < NS; ++p) {
+        float a = P.wetc[w][p][NS] * phN;
+#pragma unroll
+        for (int q = 0; q < NS; ++q) a += P.wetc[w][p][q] * ph[q];
+        sp[p] = ph[p] * a;
+    }
+#pragma unroll
+    for (int p = 0; p < NS; ++p) ph[p] += k2 * sp[p];
+}
+
+// What complete_node reads of its own node from the rings of the row march:
+// j and phi_lo (j rows of the node's row) and phi of a neighbour.
+template <int NS>
+struct OwnRing {
+    const float *s_j, *s_phi;
+    int T, t, sm, s0, sp;
+    static constexpr int NE = ring_even(NS);
+    template <class V> __device__ __forceinline__ V jx(int p) const { return rld<V>(s_j, T, p, t); }
+    template <class V> __device__ __forceinline__ V jy(int p) const { return rld<V>(s_j + NE * T, T, p, t); }
+    template <class V> __device__ __forceinline__ V plo(int p) const { return rld<V>(s_j + 2 * NE * T, T, p, t); }
+    template <class V> __device__ __forceinline__ V phi_at(int p, int cx, int cy) const
+    {
+        return rld<V>(s_phi + (cy > 0 ? sp : (cy < 0 ? sm : s0)) * NE * T, T, p, t + cx);
+    }
+};
+
+// a b + c d with the first product fused.  Left to the compiler, which of the
+// two is fused depends on the code around the sum, and the row march and the
+// patch kernel have to give the same bits.
+__device__ __forceinline__ float two_products(float a, float b, float c, float d)
+{
+    return __fmaf_rn(a, b, __fmul_rn(c, d));
+}
+
+// phi, grad phi and lap phi of all N phases from those of phases 1..N-1
+// (phase N by phi_N = 1 - sum and negated sums).
+template <int NS>
+__device__ __forceinline__ void close_phases(const float (&PH)[NS], const float (&GX)[NS], const float (&GY)[NS],
+                                             const float (&LP)[NS], float (&ph)[NS + 1], float (&gx)[NS + 1],
+                                             float (&gy)[NS + 1], float (&lap)[NS + 1])
+{
+    float sph = 0.f, sgx = 0.f, sgy = 0.f, sl = 0.f;
+#pragma unroll
+    for (int p = 0; p < NS; ++p) {
+        ph[p] = PH[p];
+        gx[p] = GX[p];
+        gy[p] = GY[p];
+        lap[p] = LP[p];
+        sph += ph[p];
+        sgx += gx[p];
+        sgy += gy[p];
+        sl += lap[p];
+    }
+    ph[NS] = 1.f - sph;
+    gx[NS] = -sgx;
+    gy[NS] = -sgy;
+    lap[NS] = -sl;
+}
+
+// Completes one node of the step: F_s and F_c, u and P, both collisions and
+// the stores.  ph, gx, gy, lap: phi and its stencils of all N phases; wm, w0,
+// wp: w = m_phi,x u_y - u_x m_phi,y at the node's column on the rows below,
+// of and above it; load_g fills the pulled g_1..g_8; php, mp: phi and m_phi
+// of the previous step; R, mph: the source and m_phi of this one; up: the
+// previous velocity; own: see OwnRing.
+template <int NS, int ST, bool TAPE, class LoadG, class Own>
+__device__ __forceinline__ void complete_node(const StepParams &P, const unsigned node, const int xg, const int y,
+                                              const float (&ph)[NS + 1], const float (&gx)[NS + 1],
+                                              const float (&gy)[NS + 1], const float (&lap)[NS + 1], const float *wm,
+                                              const float *w0, const float *wp, LoadG &&load_g,
+                                              const float (&php)[NS], const float mpx, const float mpy,
+                                              const float (&Rx)[NS], const float (&Ry)[NS], const float mphx,
+                                              const float mphy, const float upx, const float upy, const Own &own)
+{
+    constexpr int N = NS + 1;
+    const unsigned pl = P.plane;
+    // mixture density, viscosity and grad rho (Eqs. (11),(12))
+    float rho = P.rhoN, mu = P.muN, grx = 0.f, gry = 0.f;
+#pragma unroll
+    for (int p = 0; p < NS; ++p) {
+        rho += P.drho[p] * ph[p];
+        mu += P.dmu[p] * ph[p];
+        grx += P.drho[p] * gx[p];
+        gry += P.drho[p] * gy[p];
+    }
+
+    // chemical potentials (Eq. (17)) and F_s = sum_p mu_p grad phi_p
+    // (Eq. (16)); the partners q of phase p two at a time
+    float gp[N], muph[N];
+    {
+        const float2 one = vset<float2>(1.f), two = vset<float2>(2.f);
+#pragma unroll
+        for (int p = 0; p + 1 < N; p += 2) {
+            const float2 f = vget<float2>(ph, p);
+            vput(gp, p, vmul(vmul(vmul(two, f), vsub(one, f)), vfma(vset<float2>(-2.f), f, one)));
+        }
+        if (N & 1) gp[N - 1] = 2.f * ph[N - 1] * (1.f - ph[N - 1]) * (1.f - 2.f * ph[N - 1]);
+#pragma unroll
+        for (int p = 0; p < N; ++p) muph[p] = 0.f;
+#pragma unroll
+        for (int p = 0; p < N; ++p) {
+            const float2 php2 = vset<float2>(ph[p]), gpp = vset<float2>(gp[p]), lpp = vset<float2>(lap[p]);
+            int q = p + 1;
+#pragma unroll
+            for (; q + 1 < N; q += 2) {
+                const float2 sq = vadd(php2, vget<float2>(ph, q));
+                const float2 G = vmul(vmul(vmul(two, sq), vsub(one, sq)), vfma(vset<float2>(-2.f), sq, one));
+                const float2 b = make_float2(P.beta2[p][q], P.beta2[p][q + 1]);
+                const float2 k = make_float2(P.kap[p][q], P.kap[p][q + 1]);
+                // mu_p accumulates its terms in the order q, q + 1
+                // (the pairwise sum keeps the cancellation of
+                // g'(phi_p) - g'(phi_p + phi_q) where phase q is
+                // nearly absent; the adjoint's gradients depend on it)
+                const float2 tp = vfma(b, vsub(gpp, G), vmul(k, vget<float2>(lap, q)));
+                muph[p] += tp.x;
+                muph[p] += tp.y;
+                vput(muph, q, vadd(vget<float2>(muph, q), vfma(b, vsub(vget<float2>(gp, q), G), vmul(k, lpp))));
+            }
+            if (q < N) {
+                const float sq = ph[p] + ph[q];
+                const float G = 2.f * sq * (1.f - sq) * (1.f - 2.f * sq);
+                const float b = P.beta2[p][q], k = P.kap[p][q];
+                muph[p] += b * (gp[p] - G) + k * lap[q];
+                muph[q] += b * (gp[q] - G) + k * lap[p];
+            }
+        }
+    }
+    float Fx = 0.f, Fy = 0.f;
+#pragma unroll
+    for (int p = 0; p < NS; ++p) {
+        const float d = muph[p] - muph[NS];
+        Fx += d * gx[p];
+        Fy += d * gy[p];
+    }
+
+    // F_c = -div(m_phi u - u m_phi)/2 with the previous velocity:
+    // with w = m_x u_y - u_x m_y, F_c = (d_y w / 2, -d_x w / 2).
+    {
+        const float wsw = wm[-1], ws = wm[0], wse = wm[1];
+        const float ww = w0[-1], we = w0[1];
+        const float wnw = wp[-1], wn = wp[0], wne = wp[1];
+        const float dxw = (we - ww) * (1.f / 3.f) + ((wne + wse) - (wnw + wsw)) * (1.f / 12.f);
+        const float dyw = (wn - ws) * (1.f / 3.f) + ((wne + wnw) - (wse + wsw)) * (1.f / 12.f);
+        Fx += 0.5f * dyw;
+        Fy -= 0.5f * dxw;
+    }
+    // gravity: F_g = rho g (total force F = F_s + F_g + F_c)
+    Fx += rho * P.gx;
+    Fy += rho * P.gy;
+
+    // macroscopic velocity (Eq. (25b)) and mass flux (Eq. (13))
+    float g[9];
+    load_g(g);
+    const float sg = ((g[1] + g[2]) + (g[3] + g[4])) + ((g[5] + g[6]) + (g[7] + g[8]));
+    const float jgx = (g[1] - g[3]) + (g[5] - g[6]) + (g[8] - g[7]);
+    const float jgy = (g[2] - g[4]) + (g[5] + g[6]) - (g[7] + g[8]);
+    const float d58 = (g[5] + g[6]) + (g[7] + g[8]);
+    const float Pxx = (g[1] + g[3]) + d58;
+    const float Pyy = (g[2] + g[4]) + d58;
+    const float Pxy = (g[5] - g[6]) + (g[7] - g[8]);
+    const float inv_rho = 1.f / rho;
+    const float2 uv = vmul(vfma(vset<float2>(0.5f), make_float2(Fx, Fy), make_float2(jgx, jgy)),
+                           vset<float2>(inv_rho));
+    const float ux = uv.x, uy = uv.y;
+    const float2 mv = vfma(vset<float2>(rho), uv, make_float2(mphx, mphy));
+    const float mx = mv.x, my = mv.y;
+    const float ugr = ux * grx + uy * gry;
+    float rho_prev = P.rhoN;
+#pragma unroll
+    for (int p = 0; p < NS; ++p) rho_prev += P.drho[p] * php[p];
+    const float mu_t = mx * ux + my * uy;
+    const float mu_prev = (rho_prev * upx + mpx) * upx + (rho_prev * upy + mpy) * upy;
+    // Eq. (25c): P = c_s^2/(1-w0) [sum_{i!=0} g_i + u.grad rho/2
+    //   - w0 m.u/(2 c_s^2) + w0 d_t(m.u)/(4 c_s^2)], c_s^2 = 1/3, w0 = 4/9
+    const float Pr = 0.6f * (sg + 0.5f * ugr - (2.f / 3.f) * mu_t + (1.f / 3.f) * (mu_t - mu_prev));
+
+    // phase-field collisions, Eqs. (18),(19) in moment space
+    // links of this node that end in a wall: their population comes
+    // back to this node (half-way bounce-back)
+    const bool bxl = P.wall_x && xg == 0, bxh = P.wall_x && xg == P.nx - 1;
+    const bool byl = P.wall_y && y == 0, byh = P.wall_y && y == P.ny - 1;
+    auto bounce = [&](int j) {
+        return (cx_of(j) < 0 && bxl) || (cx_of(j) > 0 && bxh) || (cy_of(j) < 0 && byl) ||
+               (cy_of(j) > 0 && byh);
+    };
+    (void)bounce;
+    const CollCoef<float2> k2(P.s1, ux, uy, upx, upy);
+    const CollCoef<float> k1(P.s1, ux, uy, upx, upy);
+    auto collide = [&](auto tag, const auto &k, int p) {
+        using V = decltype(tag);
+        V A, B, C, D;
+        phase_moments<V>(vget<V>(ph, p), own.template jx<V>(p), own.template jy<V>(p), vget<V>(php, p),
+                         vget<V>(Rx, p), vget<V>(Ry, p), k, A, B, C, D);
+        if constexpr (ST == 0) {
+            V fo[9];
+            phase_populations<V>(vget<V>(ph, p), own.template plo<V>(p), A, B, C, D, fo);
+#pragma unroll
+            for (int i = 0; i < 9; ++i) vstore(P.fout + ((size_t)p * 9 + i) * pl + node, 9 * (size_t)pl, fo[i]);
+        } else {
+            // f*_j = w_j phi + h_j; stored: dev_j = f*_j - w_j phi(puller
+            // of j), rounded to 16 bits (a phase pair's two deviations
+            // in one word).  The rest population (FP32) is what makes
+            // the nine values the pullers reconstruct sum to phi.
+            const V phi = vget<V>(ph, p);
+            const V h1 = vmul(vset<V>(0.5f), vsub(A, D)), h2 = vmul(vset<V>(0.5f), vsub(B, C));
+            const V h5 = vmul(vset<V>(0.25f), vadd(C, D)), h6 = vmul(vset<V>(0.25f), vsub(C, D));
+            const V zero = vset<V>(0.f);
+            const V hdev[9] = {zero, h1, h2, vsub(zero, h1), vsub(zero, h2), h5, h6, vsub(zero, h5),
+                               vsub(zero, h6)};
+            V r[9];
+#pragma unroll
+            for (int j = 1; j < 9; ++j) {
+                const V base = bounce(j) ? phi : own.template phi_at<V>(p, cx_of(j), cy_of(j));
+                const V dev = vfma(vset<V>(w_of(j)), vsub(phi, base), hdev[j]);
+                if constexpr (sizeof(V) == 8) {
+                    const unsigned wd = Pack16<ST>::enc2(dev);
+                    ((unsigned *)P.fout)[dev_word(p / 2, j - 1, pl, node)] = wd;
+                    r[j] = vfma(vset<V>(w_of(j)), base, Pack16<ST>::dec2(wd));
+                } else {
+                    const unsigned short q = Store16<ST>::enc(dev);
+                    ((unsigned short *)P.fout)[dev_tail(NS, j - 1, pl, node)] = q;
+                    r[j] = __fmaf_rn(w_of(j), base, Store16<ST>::dec(q));
+                }
+            }
+            V e13, e24, e57, e68, ea, eb, es, e0;
+            const V s13 = two_sum_v(r[1], r[3], e13), s24 = two_sum_v(r[2], r[4], e24);
+            const V s57 = two_sum_v(r[5], r[7], e57), s68 = two_sum_v(r[6], r[8], e68);
+            const V sa = two_sum_v(s13, s24, ea), sb = two_sum_v(s57, s68, eb);
+            const V S = two_sum_v(sa, sb, es);
+            const V E = vadd(vadd(vadd(e13, e24), vadd(e57, e68)), vadd(vadd(ea, eb), es));
+            const V a0 = two_sum_v(phi, vsub(zero, S), e0);
+            const V plo = own.template plo<V>(p);
+            vstore(P.f0out + (size_t)p * pl + node, (size_t)pl, vadd(a0, vsub(vadd(e0, plo), E)));
+        }
+        vstore(P.phi + (size_t)p * pl + node, (size_t)pl, vget<V>(ph, p));
+    };
+#pragma unroll
+    for (int p = 0; p + 1 < NS; p += 2) collide(float2(), k2, p);
+    if (NS & 1) collide(0.f, k1, NS - 1);
+
+    // flow collision, Eqs. (21)-(24), tau_g from Eq. (26)
+    {
+        // (x, y) pairs: diagonal second moments (xx, yy), first
+        // moments, and (m7, m6) = (rho u_x, rho u_y)/3 + (F_x, F_y)/6
+        const float s2r = 2.f * rho / (6.f * mu + rho);   // 1/tau_g, tau_g = 3 mu/rho + 1/2
+        const float c2 = 1.f - s2r, h2 = 1.f - 0.5f * s2r;
+        const float2 u2 = make_float2(ux, uy), F2 = make_float2(Fx, Fy), gr2 = make_float2(grx, gry);
+        const float2 Qd = vmul(make_float2(mx, my), u2);   // (Qxx, Qyy)
+        const float Qxy = 0.5f * two_products(mx, uy, my, ux);
+        const float2 dQd = vsub(vmul(make_float2(mphx, mphy), u2), vmul(make_float2(mpx, mpy), make_float2(upx, upy)));
+        const float dQxy = 0.5f * (two_products(mphx, uy, mphy, ux) - two_products(mpx, upy, mpy, upx));
+        const float2 Md = vadd(vfma(vset<float2>(2.f / 3.f), vmul(u2, gr2), vfma(vset<float2>(2.f), vmul(u2, F2), dQd)),
+                               vset<float2>((1.f / 3.f) * ugr));   // (Mxx, Myy)
+        const float Mxy = two_products(ux, Fy, Fx, uy) + dQxy + (1.f / 3.f) * two_products(ux, gry, grx, uy);
+        const float2 m12 = vadd(make_float2(jgx, jgy), F2);
+        const float2 m34 = vfma(vset<float2>(c2), make_float2(Pxx, Pyy),
+                                vfma(vset<float2>(s2r), vadd(vset<float2>(Pr), Qd), vmul(vset<float2>(h2), Md)));
+        const float m5 = two_products(s2r, Qxy, c2, Pxy) + h2 * Mxy;
+        const float2 m76 = vfma(vset<float2>(rho * (1.f / 3.f)), u2, vmul(F2, vset<float2>(1.f / 6.f)));
+        const float m6 = m76.y, m7 = m76.x;
+        const float m8 = (Pr + Qd.x + Qd.y) * (1.f / 3.f) + (Md.x + Md.y) * (1.f / 6.f) - ugr * (1.f / 18.f);
+        const float2 h34 = vsub(m34, vset<float2>(m8));
+        const float2 gs12 = vmul(vset<float2>(0.5f), vadd(vsub(m12, m76), h34));
+        const float2 gs34 = vmul(vset<float2>(0.5f), vadd(vsub(m76, m12), h34));
+        const float gs[9] = {0.f, gs12.x, gs12.y, gs34.x, gs34.y,
+                             0.25f * ((m5 + m6) + (m7 + m8)),
+                             0.25f * ((m6 - m5) + (m8 - m7)),
+                             0.25f * ((m5 - m6) + (m8 - m7)),
+                             0.25f * ((m7 - m5) + (m8 - m6))};
+        if constexpr (ST == 0) {
+            float *go = P.gout + node;
+#pragma unroll
+            for (int i = 1; i < 9; ++i) go[(i - 1) * pl] = gs[i];
+        } else {
+            // stored: g*_i - 3 w_i P of this node (the puller adds it back)
+            unsigned short *go = (unsigned short *)P.gout + node;
+#pragma unroll
+            for (int i = 1; i < 9; ++i) go[(size_t)(i - 1) * pl] = Store16<ST>::enc(__fmaf_rn(-3.f * w_of(i), Pr, gs[i]));
+        }
+    }
+    P.uout[node] = ux;
+    P.uout[pl + node] = uy;
+    P.mphi[node] = mphx;
+    P.mphi[pl + node] = mphy;
+    if (P.pout) P.pout[node] = Pr;
+    if constexpr (TAPE) {
+        // the intermediate fields of this step at this node, for the
+        // adjoint: phi, j, pulled g, grad phi, lap phi, R, m_phi, w, F
+        float *tp = P.tape + node;
+#pragma unroll
+        for (int p = 0; p < NS; ++p) {
+            tp[(size_t)p * pl] = ph[p];
+            tp[(size_t)(NS + 2 * p) * pl] = own.template jx<float>(p);
+            tp[(size_t)(NS + 2 * p + 1) * pl] = own.template jy<float>(p);
+            tp[(size_t)(3 * NS + 8 + 2 * p) * pl] = gx[p];
+            tp[(size_t)(3 * NS + 9 + 2 * p) * pl] = gy[p];
+            tp[(size_t)(5 * NS + 8 + p) * pl] = lap[p];
+            tp[(size_t)(6 * NS + 8 + 2 * p) * pl] = Rx[p];
+            tp[(size_t)(6 * NS + 9 + 2 * p) * pl] = Ry[p];
+        }
+#pragma unroll
+        for (int i = 1; i < 9; ++i) tp[(size_t)(3 * NS + i - 1) * pl] = g[i];
+        tp[(size_t)(8 * NS + 8) * pl] = mphx;
+        tp[(size_t)(8 * NS + 9) * pl] = mphy;
+        tp[(size_t)(8 * NS + 10) * pl] = w0[0];
+        tp[(size_t)(8 * NS + 11) * pl] = Fx;
+        tp[(size_t)(8 * NS + 12) * pl] = Fy;
+    }
+}
+
+// w = m_phi,x u_y - u_x m_phi,y (previous velocity), with one fused product
+// (see two_products).
+__device__ __forceinline__ float flux_cross(float mx, float my, float ux, float uy)
+{
+    return __fmaf_rn(mx, uy, -__fmul_rn(ux, my));
+}
+
 // One tile of the fused step: the strip of columns [x0, x0 + T - 4) marching
 // rows [y0, y0 + TY) of the simulation described by P.  smem is the dynamic
 // shared memory of the block (step_smem_bytes gives its size).  VEC: the
@@ -1112,27 +1443,7 @@ __device__ __forceinline__ void step_tile(const StepParams &P, const int x0, con
             } else {
                 sum_pulled16<NS, ST, true>(s_F, T, t, par_cur, ph, plo, jx, jy);
             }
-            if (P.wet && (ra < 0 || ra >= P.ny)) {
-                // ghost row beyond a wetting wall (Sec. 4.2): its mirror image
-                // plus (2k - 1) s_p, s_p = phi_p sum_q (4/eps) cos theta_pq phi_q
-                // at the image node, so that the difference across the wall
-                // is s_p (n_w pointing into the wall)
-                const int w = ra < 0 ? 0 : 1;
-                const float k2 = (float)(2 * (ra < 0 ? -ra : ra - (P.ny - 1)) - 1);
-                float phN = 1.f;
-#pragma unroll
-                for (int p = 0; p < NS; ++p) phN -= ph[p];
-                float sp[NS];
-#pragma unroll
-                for (int p = 0; p < NS; ++p) {
-                    float a = P.wetc[w][p][NS] * phN;
-#pragma unroll
-                    for (int q = 0; q < NS; ++q) a += P.wetc[w][p][q] * ph[q];
-                    sp[p] = ph[p] * a;
-                }
-#pragma unroll
-                for (int p = 0; p < NS; ++p) ph[p] += k2 * sp[p];
-            }
+            if (P.wet && (ra < 0 || ra >= P.ny)) wet_ghost<NS>(P, ra, ph);
             float *prow = s_phi + a5 * NE * T;
 #pragma unroll
             for (int p = 0; p + 1 < NS; p += 2) rst(prow, T, p, t, vget<float2>(ph, p));
@@ -1196,7 +1507,7 @@ __device__ __forceinline__ void step_tile(const StepParams &P, const int x0, con
                 }
                 source_terms<NS, MODEL>(P, ph, gx, gy, Rx, Ry);
                 mass_flux<NS>(P, gx, gy, Rx, Ry, mx, my);
-                s_w[s3 * T + t] = ub_s * (mx * ub_y - ub_x * my);
+                s_w[s3 * T + t] = ub_s * flux_cross(mx, my, ub_x, ub_y);
 #pragma unroll
                 for (int p = 0; p < NS; ++p) { Rnx[p] = Rx[p]; Rny[p] = Ry[p]; }
                 Mnx = mx;
@@ -1212,304 +1523,59 @@ __device__ __forceinline__ void step_tile(const StepParams &P, const int x0, con
             const int sm = a5m3, s0 = a5m2, sp = a5m1;
             float ph[N], gx[N], gy[N], lap[N];
             if constexpr (ST == 0) {
-                float sph = 0.f, sgx = 0.f, sgy = 0.f, sl = 0.f;
-#pragma unroll
-                for (int p = 0; p < NS; ++p) {
-                    ph[p] = PHc[p];
-                    gx[p] = GXc[p];
-                    gy[p] = GYc[p];
-                    lap[p] = LPc[p];
-                    sph += ph[p];
-                    sgx += gx[p];
-                    sgy += gy[p];
-                    sl += lap[p];
-                }
-                ph[NS] = 1.f - sph;
-                gx[NS] = -sgx;
-                gy[NS] = -sgy;
-                lap[NS] = -sl;
+                close_phases<NS>(PHc, GXc, GYc, LPc, ph, gx, gy, lap);
             } else {
                 window_grad_lap<NS>(s_phi, T, sm, s0, sp, t, ph, gx, gy, lap);
             }
 
-            // mixture density, viscosity and grad rho (Eqs. (11),(12))
-            float rho = P.rhoN, mu = P.muN, grx = 0.f, gry = 0.f;
+            auto load_g = [&](float (&gv)[9]) {
+                if constexpr (V32) {
+                    const float *gw = s_Gw + (y & 1) * (T / 32) * 8 * kWin;
+                    const WinCols wcl = win_cols(2 + lane, P.wall_y && y == 0, P.wall_y && y == P.ny - 1);
+                    gv[1] = gw[wcl.b - 1];
+                    gv[2] = gw[kWin + wcl.b];
+                    gv[3] = gw[2 * kWin + wcl.b + 1];
+                    gv[4] = gw[3 * kWin + wcl.b];
+                    gv[5] = gw[4 * kWin + wcl.c5];
+                    gv[6] = gw[5 * kWin + wcl.c6];
+                    gv[7] = gw[6 * kWin + wcl.c7];
+                    gv[8] = gw[7 * kWin + wcl.c8];
+                } else if constexpr (ST == 0) {
 #pragma unroll
-            for (int p = 0; p < NS; ++p) {
-                rho += P.drho[p] * ph[p];
-                mu += P.dmu[p] * ph[p];
-                grx += P.drho[p] * gx[p];
-                gry += P.drho[p] * gy[p];
-            }
-
-            // chemical potentials (Eq. (17)) and F_s = sum_p mu_p grad phi_p
-            // (Eq. (16)); the partners q of phase p two at a time
-            float gp[N], muph[N];
-            {
-                const float2 one = vset<float2>(1.f), two = vset<float2>(2.f);
-#pragma unroll
-                for (int p = 0; p + 1 < N; p += 2) {
-                    const float2 f = vget<float2>(ph, p);
-                    vput(gp, p, vmul(vmul(vmul(two, f), vsub(one, f)), vfma(vset<float2>(-2.f), f, one)));
-                }
-                if (N & 1) gp[N - 1] = 2.f * ph[N - 1] * (1.f - ph[N - 1]) * (1.f - 2.f * ph[N - 1]);
-#pragma unroll
-                for (int p = 0; p < N; ++p) muph[p] = 0.f;
-#pragma unroll
-                for (int p = 0; p < N; ++p) {
-                    const float2 php2 = vset<float2>(ph[p]), gpp = vset<float2>(gp[p]), lpp = vset<float2>(lap[p]);
-                    int q = p + 1;
-#pragma unroll
-                    for (; q + 1 < N; q += 2) {
-                        const float2 sq = vadd(php2, vget<float2>(ph, q));
-                        const float2 G = vmul(vmul(vmul(two, sq), vsub(one, sq)), vfma(vset<float2>(-2.f), sq, one));
-                        const float2 b = make_float2(P.beta2[p][q], P.beta2[p][q + 1]);
-                        const float2 k = make_float2(P.kap[p][q], P.kap[p][q + 1]);
-                        // mu_p accumulates its terms in the order q, q + 1
-                        // (the pairwise sum keeps the cancellation of
-                        // g'(phi_p) - g'(phi_p + phi_q) where phase q is
-                        // nearly absent; the adjoint's gradients depend on it)
-                        const float2 tp = vfma(b, vsub(gpp, G), vmul(k, vget<float2>(lap, q)));
-                        muph[p] += tp.x;
-                        muph[p] += tp.y;
-                        vput(muph, q, vadd(vget<float2>(muph, q), vfma(b, vsub(vget<float2>(gp, q), G), vmul(k, lpp))));
-                    }
-                    if (q < N) {
-                        const float sq = ph[p] + ph[q];
-                        const float G = 2.f * sq * (1.f - sq) * (1.f - 2.f * sq);
-                        const float b = P.beta2[p][q], k = P.kap[p][q];
-                        muph[p] += b * (gp[p] - G) + k * lap[q];
-                        muph[q] += b * (gp[q] - G) + k * lap[p];
-                    }
-                }
-            }
-            float Fx = 0.f, Fy = 0.f;
-#pragma unroll
-            for (int p = 0; p < NS; ++p) {
-                const float d = muph[p] - muph[NS];
-                Fx += d * gx[p];
-                Fy += d * gy[p];
-            }
-
-            // F_c = -div(m_phi u - u m_phi)/2 with the previous velocity:
-            // with w = m_x u_y - u_x m_y, F_c = (d_y w / 2, -d_x w / 2).
-            {
-                const float *wm = s_w + a3 * T + t;
-                const float *w0 = s_w + a3m2 * T + t;
-                const float *wp = s_w + a3m1 * T + t;
-                const float wsw = wm[-1], ws = wm[0], wse = wm[1];
-                const float ww = w0[-1], we = w0[1];
-                const float wnw = wp[-1], wn = wp[0], wne = wp[1];
-                const float dxw = (we - ww) * (1.f / 3.f) + ((wne + wse) - (wnw + wsw)) * (1.f / 12.f);
-                const float dyw = (wn - ws) * (1.f / 3.f) + ((wne + wnw) - (wse + wsw)) * (1.f / 12.f);
-                Fx += 0.5f * dyw;
-                Fy -= 0.5f * dxw;
-            }
-            // gravity: F_g = rho g (total force F = F_s + F_g + F_c)
-            Fx += rho * P.gx;
-            Fy += rho * P.gy;
-
-            // macroscopic velocity (Eq. (25b)) and mass flux (Eq. (13))
-            if constexpr (V16) {
-                const int b = (y & 1) * (T / 32) + warp;
-                const unsigned short *gd = s_G16 + b * 8 * kWin16;
-                const float *pw = s_P16 + b * 3 * kWin;   // rows y - 1, y, y + 1
-                const bool bl = P.wall_y && y == 0, bh = P.wall_y && y == P.ny - 1;
-                const WinCols wd = win_cols(lane + o16, bl, bh), wp = win_cols(2 + lane, bl, bh);
-                gq[1] = gd[wd.b - 1];
-                gq[2] = gd[kWin16 + wd.b];
-                gq[3] = gd[2 * kWin16 + wd.b + 1];
-                gq[4] = gd[3 * kWin16 + wd.b];
-                gq[5] = gd[4 * kWin16 + wd.c5];
-                gq[6] = gd[5 * kWin16 + wd.c6];
-                gq[7] = gd[6 * kWin16 + wd.c7];
-                gq[8] = gd[7 * kWin16 + wd.c8];
-                gps[1] = pw[kWin + wp.b - 1];
-                gps[2] = pw[(bl ? kWin : 0) + wp.b];
-                gps[3] = pw[kWin + wp.b + 1];
-                gps[4] = pw[(bh ? kWin : 2 * kWin) + wp.b];
-                gps[5] = pw[(bl ? kWin : 0) + wp.c5];
-                gps[6] = pw[(bl ? kWin : 0) + wp.c6];
-                gps[7] = pw[(bh ? kWin : 2 * kWin) + wp.c7];
-                gps[8] = pw[(bh ? kWin : 2 * kWin) + wp.c8];
-            }
-            if constexpr (V32) {
-                const float *gw = s_Gw + (y & 1) * (T / 32) * 8 * kWin;
-                const WinCols wcl = win_cols(2 + lane, P.wall_y && y == 0, P.wall_y && y == P.ny - 1);
-                g[1] = gw[wcl.b - 1];
-                g[2] = gw[kWin + wcl.b];
-                g[3] = gw[2 * kWin + wcl.b + 1];
-                g[4] = gw[3 * kWin + wcl.b];
-                g[5] = gw[4 * kWin + wcl.c5];
-                g[6] = gw[5 * kWin + wcl.c6];
-                g[7] = gw[6 * kWin + wcl.c7];
-                g[8] = gw[7 * kWin + wcl.c8];
-            }
-            if constexpr (ST != 0) {
-                // g_i = 3 w_i P(source) + stored deviation
-#pragma unroll
-                for (int i = 1; i < 9; ++i) g[i] = __fmaf_rn(3.f * w_of(i), gps[i], Store16<ST>::dec(gq[i]));
-            }
-            const float sg = ((g[1] + g[2]) + (g[3] + g[4])) + ((g[5] + g[6]) + (g[7] + g[8]));
-            const float jgx = (g[1] - g[3]) + (g[5] - g[6]) + (g[8] - g[7]);
-            const float jgy = (g[2] - g[4]) + (g[5] + g[6]) - (g[7] + g[8]);
-            const float d58 = (g[5] + g[6]) + (g[7] + g[8]);
-            const float Pxx = (g[1] + g[3]) + d58;
-            const float Pyy = (g[2] + g[4]) + d58;
-            const float Pxy = (g[5] - g[6]) + (g[7] - g[8]);
-            const float inv_rho = 1.f / rho;
-            const float2 uv = vmul(vfma(vset<float2>(0.5f), make_float2(Fx, Fy), make_float2(jgx, jgy)),
-                                   vset<float2>(inv_rho));
-            const float ux = uv.x, uy = uv.y;
-            const float mphx = Mcx, mphy = Mcy;
-            const float upx = Ucx, upy = Ucy;
-            const float2 mv = vfma(vset<float2>(rho), uv, make_float2(mphx, mphy));
-            const float mx = mv.x, my = mv.y;
-            const float ugr = ux * grx + uy * gry;
-            float rho_prev = P.rhoN;
-#pragma unroll
-            for (int p = 0; p < NS; ++p) rho_prev += P.drho[p] * php[p];
-            const float mu_t = mx * ux + my * uy;
-            const float mu_prev = (rho_prev * upx + mpx) * upx + (rho_prev * upy + mpy) * upy;
-            // Eq. (25c): P = c_s^2/(1-w0) [sum_{i!=0} g_i + u.grad rho/2
-            //   - w0 m.u/(2 c_s^2) + w0 d_t(m.u)/(4 c_s^2)], c_s^2 = 1/3, w0 = 4/9
-            const float Pr = 0.6f * (sg + 0.5f * ugr - (2.f / 3.f) * mu_t + (1.f / 3.f) * (mu_t - mu_prev));
-
-            // phase-field collisions, Eqs. (18),(19) in moment space
-            const int s3 = a3m2;
-            // links of this node that end in a wall: their population comes
-            // back to this node (half-way bounce-back)
-            const bool bxl = P.wall_x && xg == 0, bxh = P.wall_x && xg == nx - 1;
-            const bool byl = P.wall_y && y == 0, byh = P.wall_y && y == P.ny - 1;
-            auto bounce = [&](int j) {
-                return (cx_of(j) < 0 && bxl) || (cx_of(j) > 0 && bxh) || (cy_of(j) < 0 && byl) ||
-                       (cy_of(j) > 0 && byh);
-            };
-            (void)bounce;
-            const CollCoef<float2> k2(P.s1, ux, uy, upx, upy);
-            const CollCoef<float> k1(P.s1, ux, uy, upx, upy);
-            const float *sjx = s_j + s3 * 3 * NE * T, *sjy = sjx + NE * T, *slo = sjy + NE * T;
-            auto collide = [&](auto tag, const auto &k, int p) {
-                using V = decltype(tag);
-                V A, B, C, D;
-                phase_moments<V>(vget<V>(ph, p), rld<V>(sjx, T, p, t), rld<V>(sjy, T, p, t), vget<V>(php, p),
-                                 vget<V>(Rcx, p), vget<V>(Rcy, p), k, A, B, C, D);
-                if constexpr (ST == 0) {
-                    V fo[9];
-                    phase_populations<V>(vget<V>(ph, p), rld<V>(slo, T, p, t), A, B, C, D, fo);
-#pragma unroll
-                    for (int i = 0; i < 9; ++i) vstore(P.fout + ((size_t)p * 9 + i) * pl + node, 9 * (size_t)pl, fo[i]);
+                    for (int i = 1; i < 9; ++i) gv[i] = g[i];
                 } else {
-                    // f*_j = w_j phi + h_j; stored: dev_j = f*_j - w_j phi(puller
-                    // of j), rounded to 16 bits (a phase pair's two deviations
-                    // in one word).  The rest population (FP32) is what makes
-                    // the nine values the pullers reconstruct sum to phi.
-                    const V phi = vget<V>(ph, p);
-                    const V h1 = vmul(vset<V>(0.5f), vsub(A, D)), h2 = vmul(vset<V>(0.5f), vsub(B, C));
-                    const V h5 = vmul(vset<V>(0.25f), vadd(C, D)), h6 = vmul(vset<V>(0.25f), vsub(C, D));
-                    const V zero = vset<V>(0.f);
-                    const V hdev[9] = {zero, h1, h2, vsub(zero, h1), vsub(zero, h2), h5, h6, vsub(zero, h5),
-                                       vsub(zero, h6)};
-                    V r[9];
-#pragma unroll
-                    for (int j = 1; j < 9; ++j) {
-                        const int sl = cy_of(j) > 0 ? sp : (cy_of(j) < 0 ? sm : s0);
-                        const V base = bounce(j) ? phi : rld<V>(s_phi + sl * NE * T, T, p, t + cx_of(j));
-                        const V dev = vfma(vset<V>(w_of(j)), vsub(phi, base), hdev[j]);
-                        if constexpr (sizeof(V) == 8) {
-                            const unsigned wd = Pack16<ST>::enc2(dev);
-                            ((unsigned *)P.fout)[dev_word(p / 2, j - 1, pl, node)] = wd;
-                            r[j] = vfma(vset<V>(w_of(j)), base, Pack16<ST>::dec2(wd));
-                        } else {
-                            const unsigned short q = Store16<ST>::enc(dev);
-                            ((unsigned short *)P.fout)[dev_tail(NS, j - 1, pl, node)] = q;
-                            r[j] = __fmaf_rn(w_of(j), base, Store16<ST>::dec(q));
-                        }
+                    if constexpr (V16) {
+                        const int b = (y & 1) * (T / 32) + warp;
+                        const unsigned short *gd = s_G16 + b * 8 * kWin16;
+                        const float *pw = s_P16 + b * 3 * kWin;   // rows y - 1, y, y + 1
+                        const bool bl = P.wall_y && y == 0, bh = P.wall_y && y == P.ny - 1;
+                        const WinCols wd = win_cols(lane + o16, bl, bh), wp = win_cols(2 + lane, bl, bh);
+                        gq[1] = gd[wd.b - 1];
+                        gq[2] = gd[kWin16 + wd.b];
+                        gq[3] = gd[2 * kWin16 + wd.b + 1];
+                        gq[4] = gd[3 * kWin16 + wd.b];
+                        gq[5] = gd[4 * kWin16 + wd.c5];
+                        gq[6] = gd[5 * kWin16 + wd.c6];
+                        gq[7] = gd[6 * kWin16 + wd.c7];
+                        gq[8] = gd[7 * kWin16 + wd.c8];
+                        gps[1] = pw[kWin + wp.b - 1];
+                        gps[2] = pw[(bl ? kWin : 0) + wp.b];
+                        gps[3] = pw[kWin + wp.b + 1];
+                        gps[4] = pw[(bh ? kWin : 2 * kWin) + wp.b];
+                        gps[5] = pw[(bl ? kWin : 0) + wp.c5];
+                        gps[6] = pw[(bl ? kWin : 0) + wp.c6];
+                        gps[7] = pw[(bh ? kWin : 2 * kWin) + wp.c7];
+                        gps[8] = pw[(bh ? kWin : 2 * kWin) + wp.c8];
                     }
-                    V e13, e24, e57, e68, ea, eb, es, e0;
-                    const V s13 = two_sum_v(r[1], r[3], e13), s24 = two_sum_v(r[2], r[4], e24);
-                    const V s57 = two_sum_v(r[5], r[7], e57), s68 = two_sum_v(r[6], r[8], e68);
-                    const V sa = two_sum_v(s13, s24, ea), sb = two_sum_v(s57, s68, eb);
-                    const V S = two_sum_v(sa, sb, es);
-                    const V E = vadd(vadd(vadd(e13, e24), vadd(e57, e68)), vadd(vadd(ea, eb), es));
-                    const V a0 = two_sum_v(phi, vsub(zero, S), e0);
-                    const V plo = rld<V>(slo, T, p, t);
-                    vstore(P.f0out + (size_t)p * pl + node, (size_t)pl, vadd(a0, vsub(vadd(e0, plo), E)));
+                    // g_i = 3 w_i P(source) + stored deviation
+#pragma unroll
+                    for (int i = 1; i < 9; ++i) gv[i] = __fmaf_rn(3.f * w_of(i), gps[i], Store16<ST>::dec(gq[i]));
                 }
-                vstore(P.phi + (size_t)p * pl + node, (size_t)pl, vget<V>(ph, p));
             };
-#pragma unroll
-            for (int p = 0; p + 1 < NS; p += 2) collide(float2(), k2, p);
-            if (NS & 1) collide(0.f, k1, NS - 1);
-
-            // flow collision, Eqs. (21)-(24), tau_g from Eq. (26)
-            {
-                // (x, y) pairs: diagonal second moments (xx, yy), first
-                // moments, and (m7, m6) = (rho u_x, rho u_y)/3 + (F_x, F_y)/6
-                const float s2r = 2.f * rho / (6.f * mu + rho);   // 1/tau_g, tau_g = 3 mu/rho + 1/2
-                const float c2 = 1.f - s2r, h2 = 1.f - 0.5f * s2r;
-                const float2 u2 = make_float2(ux, uy), F2 = make_float2(Fx, Fy), gr2 = make_float2(grx, gry);
-                const float2 Qd = vmul(make_float2(mx, my), u2);   // (Qxx, Qyy)
-                const float Qxy = 0.5f * (mx * uy + my * ux);
-                const float2 dQd = vsub(vmul(make_float2(mphx, mphy), u2), vmul(make_float2(mpx, mpy), make_float2(upx, upy)));
-                const float dQxy = 0.5f * ((mphx * uy + mphy * ux) - (mpx * upy + mpy * upx));
-                const float2 Md = vadd(vfma(vset<float2>(2.f / 3.f), vmul(u2, gr2), vfma(vset<float2>(2.f), vmul(u2, F2), dQd)),
-                                       vset<float2>((1.f / 3.f) * ugr));   // (Mxx, Myy)
-                const float Mxy = ux * Fy + Fx * uy + dQxy + (1.f / 3.f) * (ux * gry + grx * uy);
-                const float2 m12 = vadd(make_float2(jgx, jgy), F2);
-                const float2 m34 = vfma(vset<float2>(c2), make_float2(Pxx, Pyy),
-                                        vfma(vset<float2>(s2r), vadd(vset<float2>(Pr), Qd), vmul(vset<float2>(h2), Md)));
-                const float m5 = c2 * Pxy + s2r * Qxy + h2 * Mxy;
-                const float2 m76 = vfma(vset<float2>(rho * (1.f / 3.f)), u2, vmul(F2, vset<float2>(1.f / 6.f)));
-                const float m6 = m76.y, m7 = m76.x;
-                const float m8 = (Pr + Qd.x + Qd.y) * (1.f / 3.f) + (Md.x + Md.y) * (1.f / 6.f) - ugr * (1.f / 18.f);
-                const float2 h34 = vsub(m34, vset<float2>(m8));
-                const float2 gs12 = vmul(vset<float2>(0.5f), vadd(vsub(m12, m76), h34));
-                const float2 gs34 = vmul(vset<float2>(0.5f), vadd(vsub(m76, m12), h34));
-                const float gs[9] = {0.f, gs12.x, gs12.y, gs34.x, gs34.y,
-                                     0.25f * ((m5 + m6) + (m7 + m8)),
-                                     0.25f * ((m6 - m5) + (m8 - m7)),
-                                     0.25f * ((m5 - m6) + (m8 - m7)),
-                                     0.25f * ((m7 - m5) + (m8 - m6))};
-                if constexpr (ST == 0) {
-                    float *go = P.gout + node;
-#pragma unroll
-                    for (int i = 1; i < 9; ++i) go[(i - 1) * pl] = gs[i];
-                } else {
-                    // stored: g*_i - 3 w_i P of this node (the puller adds it back)
-                    unsigned short *go = (unsigned short *)P.gout + node;
-#pragma unroll
-                    for (int i = 1; i < 9; ++i) go[(size_t)(i - 1) * pl] = Store16<ST>::enc(__fmaf_rn(-3.f * w_of(i), Pr, gs[i]));
-                }
-            }
-            P.uout[node] = ux;
-            P.uout[pl + node] = uy;
-            P.mphi[node] = mphx;
-            P.mphi[pl + node] = mphy;
-            if (P.pout) P.pout[node] = Pr;
-            if constexpr (TAPE) {
-                // the intermediate fields of this step at this node, for the
-                // adjoint: phi, j, pulled g, grad phi, lap phi, R, m_phi, w, F
-                float *tp = P.tape + node;
-#pragma unroll
-                for (int p = 0; p < NS; ++p) {
-                    tp[(size_t)p * pl] = ph[p];
-                    tp[(size_t)(NS + 2 * p) * pl] = rld<float>(sjx, T, p, t);
-                    tp[(size_t)(NS + 2 * p + 1) * pl] = rld<float>(sjy, T, p, t);
-                    tp[(size_t)(3 * NS + 8 + 2 * p) * pl] = gx[p];
-                    tp[(size_t)(3 * NS + 9 + 2 * p) * pl] = gy[p];
-                    tp[(size_t)(5 * NS + 8 + p) * pl] = lap[p];
-                    tp[(size_t)(6 * NS + 8 + 2 * p) * pl] = Rcx[p];
-                    tp[(size_t)(6 * NS + 9 + 2 * p) * pl] = Rcy[p];
-                }
-#pragma unroll
-                for (int i = 1; i < 9; ++i) tp[(size_t)(3 * NS + i - 1) * pl] = g[i];
-                tp[(size_t)(8 * NS + 8) * pl] = mphx;
-                tp[(size_t)(8 * NS + 9) * pl] = mphy;
-                tp[(size_t)(8 * NS + 10) * pl] = s_w[a3m2 * T + t];
-                tp[(size_t)(8 * NS + 11) * pl] = Fx;
-                tp[(size_t)(8 * NS + 12) * pl] = Fy;
-            }
+            const OwnRing<NS> own_node{s_j + a3m2 * 3 * NE * T, s_phi, T, t, sm, s0, sp};
+            complete_node<NS, ST, TAPE>(P, node, xg, y, ph, gx, gy, lap, s_w + a3 * T + t, s_w + a3m2 * T + t,
+                                        s_w + a3m1 * T + t, load_g, php, mpx, mpy, Rcx, Rcy, Mcx, Mcy, Ucx, Ucy,
+                                        own_node);
         }
 #pragma unroll
         for (int p = 0; p < NS; ++p) {
@@ -1612,34 +1678,36 @@ cudaError_t variant_slots(int dev, int *out)
     return cudaSuccess;
 }
 
+// Automatic march length: as many row chunks per strip as there are
+// resident-block slots per strip (one full wave), chunks of at least 2 rows.
+// Every chunk, of a narrow last strip too, gets the same rows: a block's
+// time per row hardly depends on how many of its warps hold ring columns.
+inline int march_chunks(const StepParams &p, int T, int nslots)
+{
+    const int strips = (p.nx + T - 5) / (T - 4);
+    const int most = p.ny / 2 > 1 ? p.ny / 2 : 1;
+    const int chunks = nslots / strips < most ? nslots / strips : most;
+    return chunks < 1 ? 1 : chunks;
+}
+
 template <int NS, int MODEL, int T, int ST, bool VEC, bool TAPE = false>
 cudaError_t launch_step_variant(const StepParams &p, int ty, int nslots, cudaStream_t st)
 {
     constexpr size_t smem = step_smem_bytes<NS, T, ST, VEC>();
     const int strips = (p.nx + T - 5) / (T - 4);
-    int chunks;
-    if (ty > 0) {
-        chunks = (p.ny + ty - 1) / ty;
-    } else {
-        // Automatic march length: as many row chunks per strip as there are
-        // resident-block slots per strip (one full wave), chunks of at least
-        // 2 rows.  On a lattice too small to fill the GPU, short chunks put
-        // more SMs to work although each repeats the 4 + 2 pre-roll rows
-        // (measured: 256^2 N=5 at 2 rows 3,188 MLUPS, at 16 rows 1,675).
-        // Every chunk, of a narrow last strip too, gets the same rows: a
-        // block's time per row hardly depends on how many of its warps hold
-        // ring columns.
-        chunks = nslots / strips;
-        const int maxc = p.ny / 2 > 1 ? p.ny / 2 : 1;
-        if (chunks > maxc) chunks = maxc;
-        if (chunks < 1) chunks = 1;
-        ty = 0;
-    }
+    const int chunks = ty > 0 ? (p.ny + ty - 1) / ty : march_chunks(p, T, nslots);
+    if (ty < 0) ty = 0;
     const long long blocks = (long long)strips * chunks;
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
     return launch_pdl(step_kernel<NS, MODEL, T, ST, VEC, TAPE>, dim3((unsigned)blocks), dim3(T), smem, st, p, ty,
                       chunks, strips);
 }
+
+}  // namespace nlbm
+
+#include "step_patch.cuh"
+
+namespace nlbm {
 
 // Row windows need nx a multiple of 4 (of 8 with 16-bit storage: rows and
 // planes start on 16-byte boundaries), 16-byte aligned arrays and no wall
@@ -1655,21 +1723,19 @@ cudaError_t launch_step_nst(const StepParams &p, int ty, cudaStream_t st)
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    {
-        uintptr_t a = reinterpret_cast<uintptr_t>(p.fin) | reinterpret_cast<uintptr_t>(p.gin);
-        if (ST != 0)
-            a |= reinterpret_cast<uintptr_t>(p.f0in) | reinterpret_cast<uintptr_t>(p.phi_prev) |
-                 reinterpret_cast<uintptr_t>(p.pin);
-        const bool vec = !p.wall_x && p.nx % (ST == 0 ? 4 : 8) == 0 && (a & 15) == 0;
-        if (vec) {
-            int win = 0;
-            if ((e = variant_slots<NS, MODEL, T, ST, true, TAPE>(dev, &win)) != cudaSuccess) return e;
-            return launch_step_variant<NS, MODEL, T, ST, true, TAPE>(p, ty, win, st);
-        }
-    }
-    int plain = 0;
-    if ((e = variant_slots<NS, MODEL, T, ST, false, TAPE>(dev, &plain)) != cudaSuccess) return e;
-    return launch_step_variant<NS, MODEL, T, ST, false, TAPE>(p, ty, plain, st);
+    uintptr_t a = reinterpret_cast<uintptr_t>(p.fin) | reinterpret_cast<uintptr_t>(p.gin);
+    if (ST != 0)
+        a |= reinterpret_cast<uintptr_t>(p.f0in) | reinterpret_cast<uintptr_t>(p.phi_prev) |
+             reinterpret_cast<uintptr_t>(p.pin);
+    const bool vec = !p.wall_x && p.nx % (ST == 0 ? 4 : 8) == 0 && (a & 15) == 0;
+    int slots = 0;
+    e = vec ? variant_slots<NS, MODEL, T, ST, true, TAPE>(dev, &slots)
+            : variant_slots<NS, MODEL, T, ST, false, TAPE>(dev, &slots);
+    if (e != cudaSuccess) return e;
+    if (ty <= 0 && use_patches<NS, ST>(p.ny, march_chunks(p, T, slots)))
+        return launch_patches<NS, MODEL, ST, TAPE>(p, st);
+    return vec ? launch_step_variant<NS, MODEL, T, ST, true, TAPE>(p, ty, slots, st)
+               : launch_step_variant<NS, MODEL, T, ST, false, TAPE>(p, ty, slots, st);
 }
 
 template <int NS, int MODEL, int ST>
