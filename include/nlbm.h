@@ -200,10 +200,11 @@ int64_t nlbm_kernel_launches(const nlbm_sim *s);
 
 /* Tile of the fused step kernel: tx threads per block (64, 128 or 256; one
  * thread per column, each block updating a strip of tx - 4 columns) marching
- * down ty rows (>= 1), or ty = 0 (the default) to let the library cut every
- * strip into equal row chunks (at least 2 rows) so that the grid is one
- * wave of resident blocks.  EINVAL outside those values.  Takes effect on
- * the next nlbm_step(). */
+ * down ty rows (>= 1), or ty = 0 (the default) to let the library choose:
+ * patches of 16 or 32 columns and 8 rows where marches would be short, else
+ * every strip cut into equal row chunks (at least 2 rows) so that the grid
+ * is one wave of resident blocks.  Results do not depend on the tile.
+ * EINVAL outside those values.  Takes effect on the next nlbm_step(). */
 nlbm_status nlbm_set_tile(nlbm_sim *s, int32_t tx, int32_t ty);
 nlbm_status nlbm_get_tile(const nlbm_sim *s, int32_t *tx, int32_t *ty);
 
@@ -264,9 +265,9 @@ nlbm_status nlbm_phase_mass_noalloc(const float *dev_phi, int32_t n_phases, int6
  * viscosities, surface tensions, epsilon and mobility -- the kind of sweep
  * the paper runs case by case (the Model A exponents of Sec. 4, the lens
  * tension ratios of Sec. 4.3, Table 3).  Members share N and FP32 storage.
- * One persistent kernel launch per step advances every member: the blocks
- * resident on the GPU take (member, column strip, row chunk) tiles from a
- * table ordered largest member first.  Steps of nlbm_batch_step() are
+ * One kernel launch per step advances every member: blocks take (member,
+ * patch) or (member, column strip, row chunk) tiles from a table ordered
+ * largest member first.  Steps of nlbm_batch_step() are
  * replayed from a captured two-step CUDA graph when the stream is not the
  * legacy default stream.  Members never exchange data.
  * ------------------------------------------------------------------------ */
@@ -297,9 +298,12 @@ nlbm_status nlbm_batch_step(nlbm_batch *b, int64_t nsteps);
 nlbm_status nlbm_batch_get_moments(nlbm_batch *b, int32_t sim, float *dev_phi, float *dev_u, float *dev_p);
 nlbm_status nlbm_batch_phase_mass(nlbm_batch *b, int32_t sim, double *host_mass);
 
-/* Tile shape of the ensemble kernel: tx threads per block (64, 128, 256;
- * strips of tx - 4 columns) and ty rows per tile (>= 1, 0 = 32).  Rebuilds
- * the tile table (synchronizes).  get_tile also returns the tile count. */
+/* Tile shape of the ensemble kernel: tx threads per block (64, 128, 256) and
+ * ty rows per tile (>= 1): strips of tx - 4 columns marched down ty rows, or,
+ * with 128 or 256 threads and ty = 8, patches of tx / 8 columns computed at
+ * once; ty = 0 (the default) lets the library choose (patches of 32 columns).
+ * Results do not depend on the shape.  Rebuilds the tile table
+ * (synchronizes).  get_tile also returns the tile count. */
 nlbm_status nlbm_batch_set_tile(nlbm_batch *b, int32_t tx, int32_t ty);
 nlbm_status nlbm_batch_get_tile(const nlbm_batch *b, int32_t *tx, int32_t *ty, int32_t *ntiles);
 

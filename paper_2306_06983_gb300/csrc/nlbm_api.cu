@@ -636,12 +636,29 @@ struct BatchLayout {
     std::vector<size_t> sim_off;
 };
 
-// Largest number of tiles any allowed tile shape gives (tx = 64, ty = 1).
+// Largest number of tiles any allowed tile shape gives (tx = 64, ty = 1, or
+// patches of 16 x 8 on a lattice of few rows).
 size_t worst_tiles(const nlbm_params *p, int count)
 {
     size_t t = 0;
-    for (int k = 0; k < count; ++k) t += (size_t)((p[k].nx + 59) / 60) * (size_t)p[k].ny;
+    for (int k = 0; k < count; ++k)
+        t += std::max((size_t)((p[k].nx + 59) / 60) * (size_t)p[k].ny,
+                      (size_t)((p[k].nx + 15) / 16) * (size_t)((p[k].ny + 7) / 8));
     return t;
+}
+
+// Columns of the ensemble's patches (of 8 rows), 0 where it marches rows:
+// with the library's own choice (ty = 0) wide patches, and tiles of 8 rows
+// are patches of tx threads.  Members are small, so a march repeats its 6
+// pre-roll rows often and its last strip is narrow (us a step, march 128 x 32
+// / best march / narrow / wide patches: 64 lenses of 512 x 256 to 128 x 64,
+// N = 3, 228 / 215 / 233 / 195; 8 of them 78 / 44 / 38 / 33; 32 members N = 5
+// 304 / 292 / 260 / 250; 16 members N = 8 413 / 331 / 253 / 242; four of
+// 1024^2, N = 5 406 / 397 / 406 / 399).
+int batch_patch_columns(int tx, int ty)
+{
+    if (ty == 0) return 32;
+    return ty == 8 && tx > 64 ? tx / 8 : 0;
 }
 
 nlbm_status batch_layout(const nlbm_params *p, int count, BatchLayout *B, char *err)
@@ -695,7 +712,7 @@ nlbm_status batch_fail(nlbm_batch *b, cudaError_t e, const char *what)
 // simulation, the largest simulations first (so the last tiles are small).
 nlbm_status build_tiles(nlbm_batch *b)
 {
-    const int W = b->tx - 4;
+    const int px = batch_patch_columns(b->tx, b->ty), W = px ? px : b->tx - 4;
     std::vector<int> order(b->count);
     for (int k = 0; k < b->count; ++k) order[k] = k;
     std::stable_sort(order.begin(), order.end(), [&](int a, int c) {
@@ -705,7 +722,7 @@ nlbm_status build_tiles(nlbm_batch *b)
     for (int k : order) {
         const nlbm_sim *s = b->sims[k];
         const int nx = s->kp.nx, ny = s->kp.ny;
-        int ty = b->ty > 0 ? b->ty : 32;
+        int ty = px ? 8 : b->ty;
         if (ty > ny) ty = ny;
         for (int y0 = 0; y0 < ny; y0 += ty)
             for (int x0 = 0; x0 < nx; x0 += W) t.push_back(BatchTile{k, x0, y0, ty});
@@ -749,6 +766,8 @@ nlbm_status upload_params(nlbm_batch *b)
 cudaError_t batch_launch(nlbm_batch *b, int parity, bool with_p)
 {
     const StepParams *tab = b->d_params + (size_t)(2 * parity + (with_p ? 1 : 0)) * b->count;
+    const int px = batch_patch_columns(b->tx, b->ty);
+    if (px) return launch_batch_patches(b->ns, px, tab, b->d_tiles, b->ntiles, b->d_counters, parity, b->stream);
     return launch_batch_step(b->ns, b->tx, tab, b->d_tiles, b->ntiles, b->d_counters, parity, b->stream);
 }
 

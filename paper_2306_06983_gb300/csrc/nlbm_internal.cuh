@@ -136,6 +136,11 @@ cudaError_t launch_step_tape_b_f32(int ns, const StepParams &p, cudaStream_t st)
 cudaError_t launch_batch_step(int ns, int tx, const StepParams *d_params, const BatchTile *d_tiles,
                               int ntiles, int *d_counters, int parity, cudaStream_t st);
 
+// The same on patches of px x 8 nodes (px = 16 or 32): d_tiles lists patches
+// and every patch is one block.
+cudaError_t launch_batch_patches(int ns, int px, const StepParams *d_params, const BatchTile *d_tiles, int ntiles,
+                                 int *d_counters, int parity, cudaStream_t st);
+
 // Auxiliary kernels (aux_kernels.cu).
 cudaError_t launch_init(int ns, const StepParams &p, cudaStream_t st);
 // A state in motion (velocity.cu): p describes the state set by launch_init

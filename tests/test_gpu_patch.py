@@ -60,3 +60,25 @@ def test_patches_equal_marches_wetting_walls(storage):
     p, phi0 = W.compound_droplet(60.0, nx=100, ny=50, R=20.0)
     p = dict(p, storage=storage, wall_cos=[0.3, 0.5, -0.2, 0.1])
     assert state(p, phi0, None) == state(p, phi0, (128, 7))
+
+
+@pytest.mark.parametrize("N", [2, 3, 4, 5, 6, 8])
+def test_ensemble_patches_equal_marches(N):
+    """Members smaller than a patch, on and off its edges, of both models;
+    patches of either width and marches, switched between steps (a march
+    after patches needs its tile counter)."""
+    from paper_2306_06983_gb300.nlbm import Batch
+    mem = [W.random_smooth(nx, ny, N, seed=N + nx, model=m, wall_x=wx, wall_y=wy, n_disks=3)
+           for nx, ny, m, wx, wy in ((17, 1, "B", False, False), (33, 9, "A", False, True), (64, 48, "B", False, False),
+                                     (45, 30, "A", True, True), (100, 40, "B", False, True))]
+    out = []
+    for tiles in (((64, 5),) * 3, ((128, 0),) * 3, ((128, 8), (64, 5), (256, 8))):
+        b = Batch([p for p, _ in mem])
+        for k, (_, phi0) in enumerate(mem):
+            b.set_phi(k, phi0.astype(np.float32))
+        for tx, ty in tiles:
+            b.set_tile(tx, ty)
+            b.step(3)
+        out.append([t.cpu().numpy().tobytes() for k in range(len(mem)) for t in b.moments(k)])
+        b.close()
+    assert out[0] == out[1] == out[2]
