@@ -15,11 +15,20 @@
 //   rev3  transposes of the isotropic gradient and Laplacian (Eq. (27));
 //   rev4  transpose of the pull (streaming) and of the moments
 //         phi = sum f_i, j = sum c_i f_i (Eq. (25a)).
+// A sweep runs them as two launches a step: rev4 of the following step and
+// rev1 (rev_collide_kernel: the adjoints of the populations are gathered
+// where they are used and never stored, 208 bytes a node less at N = 3), and
+// rev2 and rev3 (rev_source_kernel).  Against one launch per pass, per-node
+// FP64 gradient sums and the same taping rebuild: 1024^2 N = 3 (Model B)
+// backward 249 -> 211 us a step, 256^2 24.1 -> 20.4.  The collision pass
+// moves 4.0 TB/s of DRAM traffic at 24 warps an SM (80 registers) and 39 %
+// issue; more loads in flight (its inputs staged by cp.async) did not change
+// its time, nor did precomputed neighbour offsets.
 // The adjoint of the step's inputs is the seed of the previous step.  The
 // derivatives are those of the exact-arithmetic step; the exact-sum devices
 // of the forward kernel (compensated sums, paired populations) change only
-// rounding.  Per-node contributions to dL/d sigma_pq and dL/dM are summed
-// in FP64 in a fixed order each step.
+// rounding.  Contributions to dL/d sigma_pq and dL/dM are summed in FP64 in a
+// fixed order: a block's nodes each step, the blocks at the end.
 #include "nlbm_internal.cuh"
 #include "adjoint.cuh"
 
@@ -33,6 +42,11 @@ __constant__ int aCy[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
 __device__ __forceinline__ float wgt(int i) { return i == 0 ? 4.f / 9.f : (i < 5 ? 1.f / 9.f : 1.f / 36.f); }
 
 __constant__ int aOpp[9] = {0, 3, 4, 1, 2, 7, 8, 5, 6};
+
+// Direction vectors and opposites that fold to constants in unrolled loops.
+__device__ __forceinline__ int cxi(int i) { return (i == 1 || i == 5 || i == 8) ? 1 : (i == 3 || i == 6 || i == 7) ? -1 : 0; }
+__device__ __forceinline__ int cyi(int i) { return (i == 2 || i == 5 || i == 6) ? 1 : (i == 4 || i == 7 || i == 8) ? -1 : 0; }
+__device__ __forceinline__ int oppi(int i) { return i == 0 ? 0 : (i < 5 ? (i + 1) % 4 + 1 : (i - 3) % 4 + 5); }
 
 __device__ __forceinline__ unsigned wrap_node(int x, int y, int nx, int ny)
 {
@@ -322,12 +336,29 @@ __global__ void tape_force_kernel(const StepParams P, AdjTape T)
 // rev1: pointwise adjoint of the collisions and everything between the
 // tape fields and them.  Seeds at x: A.lf_out (f*), A.lg_out (g*), A.lphi_out
 // (phi(t): the next step's phi_prev and the loss), A.lu_out, A.lm_out.
-template <int NS>
-__device__ __forceinline__ void rev_collide_node(const StepParams &P, const AdjTape &T, const AdjFields &A, unsigned k)
+//
+// GATHER: the seeds of the populations are not fields but are taken here from
+// the following step's adjoints of phi, j and the pulled g, the transpose of
+// its pull: f*_i of this step at x was pulled at x + c_i (or, where that is
+// beyond a wall, at x itself as direction opp(i)) and entered phi and j there.
+// Returns the node's dL/dsigma_pq and dL/dM terms in sums.
+template <int NS, bool GATHER, bool WALLS>
+__device__ __forceinline__ void rev_collide_node(const StepParams &P, const AdjTape &T, const AdjFields &A, const int x,
+                                                 const int y, const unsigned k,
+                                                 float (&sums)[(NS + 1) * NS / 2 + 1])
 {
     constexpr int N = NS + 1;
     constexpr int NP = N * (N - 1) / 2;
     const unsigned pl = P.plane;
+    unsigned pn[9];    // GATHER: node that pulled f*_i of this node
+    bool pb[9];        // ... bounced back
+    if constexpr (GATHER) {
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            pb[i] = WALLS && beyond_wall(P, x + cxi(i), y + cyi(i));
+            pn[i] = pb[i] ? k : wrap_node(x + cxi(i), y + cyi(i), P.nx, P.ny);
+        }
+    }
     {
         // ---------------- forward values at x
         float ph[N], lap[N], gx[NS], gy[NS], jx[NS], jy[NS], Rx[NS], Ry[NS], php[NS];
@@ -353,9 +384,6 @@ __device__ __forceinline__ void rev_collide_node(const StepParams &P, const AdjT
         }
         ph[NS] = 1.f - sph;
         lap[NS] = -sl;
-        double gacc[NP + 1];   // updated at the end; loaded before the first store
-#pragma unroll
-        for (int q = 0; q <= NP; ++q) gacc[q] = A.gacc[(size_t)q * pl + k];
         float g[9];
 #pragma unroll
         for (int i = 1; i < 9; ++i) g[i] = __ldg(T.g + (size_t)(i - 1) * pl + k);
@@ -400,7 +428,10 @@ __device__ __forceinline__ void rev_collide_node(const StepParams &P, const AdjT
         // ---------------- flow collision (Eqs. (21)-(24)) reversed
         float lg[9];
 #pragma unroll
-        for (int i = 1; i < 9; ++i) lg[i] = __ldg(A.lg_out + (size_t)(i - 1) * pl + k);
+        for (int i = 1; i < 9; ++i) {
+            if constexpr (GATHER) lg[i] = __ldg(A.lg_next + (size_t)((pb[i] ? oppi(i) : i) - 1) * pl + pn[i]);
+            else lg[i] = __ldg(A.lg_out + (size_t)(i - 1) * pl + k);
+        }
         const float a_m1 = 0.5f * (lg[1] - lg[3]);
         const float a_m2 = 0.5f * (lg[2] - lg[4]);
         const float a_m3 = 0.5f * (lg[1] + lg[3]);
@@ -476,7 +507,23 @@ __device__ __forceinline__ void rev_collide_node(const StepParams &P, const AdjT
         for (int p = 0; p < NS; ++p) {
             float lf[9];
 #pragma unroll
-            for (int i = 0; i < 9; ++i) lf[i] = __ldg(A.lf_out + ((size_t)p * 9 + i) * pl + k);
+            for (int i = 0; i < 9; ++i) {
+                if constexpr (GATHER) {
+                    // lphi + c . lj, c = c_i, or -c_i for a bounced link
+                    float v = __ldg(A.lphi_tot + (size_t)p * pl + pn[i]);
+                    if (cxi(i) != 0) {
+                        const float j = __ldg(A.lj_next + (size_t)(2 * p) * pl + pn[i]);
+                        v += ((cxi(i) > 0) != pb[i]) ? j : -j;
+                    }
+                    if (cyi(i) != 0) {
+                        const float j = __ldg(A.lj_next + (size_t)(2 * p + 1) * pl + pn[i]);
+                        v += ((cyi(i) > 0) != pb[i]) ? j : -j;
+                    }
+                    lf[i] = v;
+                } else {
+                    lf[i] = __ldg(A.lf_out + ((size_t)p * 9 + i) * pl + k);
+                }
+            }
             const float phi = ph[p];
             const float Gx = 3.f * (phi * ux - php[p] * upx) + Rx[p];
             const float Gy = 3.f * (phi * uy - php[p] * upy) + Ry[p];
@@ -573,7 +620,6 @@ __device__ __forceinline__ void rev_collide_node(const StepParams &P, const AdjT
             a_gx[p] += d * a_Fx;
             a_gy[p] += d * a_Fy;
         }
-        float dsig[NP > 0 ? NP : 1];
         int pair = 0;
 #pragma unroll
         for (int p = 0; p < N; ++p)
@@ -588,7 +634,7 @@ __device__ __forceinline__ void rev_collide_node(const StepParams &P, const AdjT
                 a_lap[p] += kq * a_muc[q];
                 // beta2 = 6 sigma / eps, kap = 3 eps sigma / 4
                 const float G1 = gp1(s);
-                dsig[pair++] = a_muc[p] * (P.six_over_eps * (gp1(ph[p]) - G1) + P.three_eps_over_4 * lap[q]) +
+                sums[pair++] = a_muc[p] * (P.six_over_eps * (gp1(ph[p]) - G1) + P.three_eps_over_4 * lap[q]) +
                                a_muc[q] * (P.six_over_eps * (gp1(ph[q]) - G1) + P.three_eps_over_4 * lap[p]);
             }
         // phase N = 1 - sum: fold its adjoints onto phases 1..N-1
@@ -617,24 +663,24 @@ __device__ __forceinline__ void rev_collide_node(const StepParams &P, const AdjT
         A.lu_in[pl + k] = a_upy;
         A.lm_in[k] = a_mpx;
         A.lm_in[pl + k] = a_mpy;
-#pragma unroll
-        for (int q = 0; q < NP; ++q) A.gacc[(size_t)q * pl + k] = gacc[q] + (double)dsig[q];
         // s1 = 1 / (1/2 + 3 M): d s1 / dM = -3 s1^2
-        A.gacc[(size_t)NP * pl + k] = gacc[NP] + (double)(-3.f * s1 * s1 * a_s1);
+        sums[NP] = -3.f * s1 * s1 * a_s1;
     }
 }
 
 
 // rev2: F_c's stencil transposed (gather of the F adjoint at the
-// neighbours), then w, m_phi and the source (Model A or B) at the node.
+// neighbours), then w, m_phi and the source (Model A or B) at the node: what
+// they add to the adjoints of phi (d_ph), grad phi (l_gx, l_gy, which hold
+// the pointwise part of rev1 already), u(t-1) (d_ux, d_uy) and M (d_M).
 template <int NS, int MODEL, bool WALLS>
-__device__ __forceinline__ void rev_source_node(const StepParams &P, const AdjTape &T, const AdjFields &A, unsigned k)
+__device__ __forceinline__ void rev_source_node(const StepParams &P, const AdjTape &T, const AdjFields &A, const int x,
+                                                const int y, const unsigned k, float (&d_ph)[NS], float (&l_gx)[NS],
+                                                float (&l_gy)[NS], float &d_ux, float &d_uy, float &d_M)
 {
     constexpr int N = NS + 1;
-    constexpr int NP = N * (N - 1) / 2;
     const unsigned pl = P.plane;
     {
-        const int x = k % P.nx, y = k / P.nx;
         // F_c(x) = (1/2 d_y w, -1/2 d_x w): w at position z enters F_c(z -
         // c_i) with weight 3 w_i c_i; the positions holding this node's w
         // are the node and, next to a wall, its ghosts (w there formed from
@@ -670,16 +716,9 @@ __device__ __forceinline__ void rev_source_node(const StepParams &P, const AdjTa
         // w = s1 mx uy + s2 ux my (previous velocity)
         const float a_mx = __ldg(A.lmphi + k) + a_ws1 * upy;
         const float a_my = __ldg(A.lmphi + pl + k) + a_ws2 * upx;
-        // the values this pass updates, loaded before its first store (the
-        // compiler may not move a load across a store to another field)
-        const float lux = A.lu_in[k], luy = A.lu_in[pl + k];
-        const double gM = A.gacc[(size_t)NP * pl + k];
-        float pw[NS];
-#pragma unroll
-        for (int p = 0; p < NS; ++p) pw[p] = A.lphi_pw[(size_t)p * pl + k];
         // m_phi = -M sum_p drho_p (grad phi_p - R_p)
         float ph[N], gx[N], gy[N], a_ph[N], a_gx[N], a_gy[N], a_Rx[NS], a_Ry[NS];
-        float sph = 0.f, sgx = 0.f, sgy = 0.f, dM = 0.f;
+        float sph = 0.f, sgx = 0.f, sgy = 0.f;
 #pragma unroll
         for (int p = 0; p < NS; ++p) {
             ph[p] = __ldg(T.phi + (size_t)p * pl + k);
@@ -689,12 +728,10 @@ __device__ __forceinline__ void rev_source_node(const StepParams &P, const AdjTa
             sgx += gx[p];
             sgy += gy[p];
             a_ph[p] = 0.f;
-            a_gx[p] = A.lgrad[(size_t)(2 * p) * pl + k] - P.mob * P.drho[p] * a_mx;
-            a_gy[p] = A.lgrad[(size_t)(2 * p + 1) * pl + k] - P.mob * P.drho[p] * a_my;
+            a_gx[p] = __ldg(A.lgrad + (size_t)(2 * p) * pl + k) - P.mob * P.drho[p] * a_mx;
+            a_gy[p] = __ldg(A.lgrad + (size_t)(2 * p + 1) * pl + k) - P.mob * P.drho[p] * a_my;
             a_Rx[p] = __ldg(A.lR + (size_t)(2 * p) * pl + k) + P.mob * P.drho[p] * a_mx;
             a_Ry[p] = __ldg(A.lR + (size_t)(2 * p + 1) * pl + k) + P.mob * P.drho[p] * a_my;
-            const float Rx = __ldg(T.R + (size_t)(2 * p) * pl + k), Ry = __ldg(T.R + (size_t)(2 * p + 1) * pl + k);
-            dM -= P.drho[p] * ((gx[p] - Rx) * a_mx + (gy[p] - Ry) * a_my);
         }
         ph[NS] = 1.f - sph;
         gx[NS] = -sgx;
@@ -774,60 +811,20 @@ __device__ __forceinline__ void rev_source_node(const StepParams &P, const AdjTa
         }
 #pragma unroll
         for (int p = 0; p < NS; ++p) {
-            A.lphi_pw[(size_t)p * pl + k] = pw[p] + (a_ph[p] - a_ph[NS]);
-            A.lgrad[(size_t)(2 * p) * pl + k] = a_gx[p] - a_gx[NS];
-            A.lgrad[(size_t)(2 * p + 1) * pl + k] = a_gy[p] - a_gy[NS];
+            d_ph[p] = a_ph[p] - a_ph[NS];
+            l_gx[p] = a_gx[p] - a_gx[NS];
+            l_gy[p] = a_gy[p] - a_gy[NS];
         }
-        A.lu_in[k] = lux + a_ws2 * mphy;
-        A.lu_in[pl + k] = luy + a_ws1 * mphx;
-        A.gacc[(size_t)NP * pl + k] = gM + (double)dM;
+        d_ux = a_ws2 * mphy;
+        d_uy = a_ws1 * mphx;
+        // dm_phi/dM = -sum_p drho_p (grad phi_p - R_p) = m_phi / M
+        d_M = (mphx * a_mx + mphy * a_my) / P.mob;
     }
 }
 
-
-// rev3: the gradient and Laplacian stencils transposed: phi_p(z) entered
-// grad phi_p(z - c_i) with weight 3 w_i c_i and lap phi_p(z - c_i) with 6 w_i
-// (and lap phi_p(z) with -6 (1 - w_0)).
-template <int NS, bool WALLS>
-__device__ __forceinline__ void rev_stencil_node(const StepParams &P, const AdjFields &A, unsigned k)
-{
-    const unsigned pl = P.plane;
-    {
-        const int x = k % P.nx, y = k / P.nx;
-#pragma unroll
-        for (int p = 0; p < NS; ++p) {
-            const float *lgx = A.lgrad + (size_t)(2 * p) * pl, *lgy = A.lgrad + (size_t)(2 * p + 1) * pl;
-            const float *ll = A.llap + (size_t)p * pl;
-            float a = __ldg(A.lphi_pw + (size_t)p * pl + k) - 6.f * (1.f - 4.f / 9.f) * __ldg(ll + k);
-            if constexpr (!WALLS) {
-#pragma unroll
-                for (int i = 1; i < 9; ++i) {
-                    const unsigned n = wrap_node(x - aCx[i], y - aCy[i], P.nx, P.ny);
-                    a += 3.f * wgt(i) * (aCx[i] * __ldg(lgx + n) + aCy[i] * __ldg(lgy + n)) + 6.f * wgt(i) * __ldg(ll + n);
-                }
-            } else {
-                // phi of this node also stands at its ghosts beyond the walls
-                int px[9], py[9];
-                const int ns = standins(P, x, y, px, py);
-                for (int s = 0; s < ns; ++s)
-#pragma unroll
-                    for (int i = 1; i < 9; ++i) {
-                        const int zx = px[s] - aCx[i], zy = py[s] - aCy[i];
-                        if (beyond_wall(P, zx, zy)) continue;
-                        const unsigned n = wrap_node(zx, zy, P.nx, P.ny);
-                        a += 3.f * wgt(i) * (aCx[i] * __ldg(lgx + n) + aCy[i] * __ldg(lgy + n)) +
-                             6.f * wgt(i) * __ldg(ll + n);
-                    }
-            }
-            A.lphi_tot[(size_t)p * pl + k] = a;
-        }
-    }
-}
-
-
-// rev4: the pull and the moments transposed.  f_i(z) = f*_i(z - c_i) fed
-// phi(z) and j(z): the adjoint of f*_i at y is lphi(y + c_i) + c_i . lj(y + c_i);
-// likewise for the flow populations.  The results seed the previous step.
+// The pull and the moments transposed as fields of their own (a single
+// reverse step returns them): the adjoint of f*_i at y is lphi(y + c_i) +
+// c_i . lj(y + c_i); likewise for the flow populations.
 template <int NS, bool WALLS>
 __device__ __forceinline__ void rev_pull_node(const StepParams &P, const AdjFields &A, unsigned k)
 {
@@ -851,45 +848,140 @@ __device__ __forceinline__ void rev_pull_node(const StepParams &P, const AdjFiel
     }
 }
 
+// The reverse passes run on tiles of 32 x 8 nodes, one node per thread, so
+// that the neighbours they gather from are mostly the block's own lines.
+constexpr int kRevX = 32, kRevY = 8, kRevThreads = kRevX * kRevY;
 
-// Threads per block of the reverse passes (one node per thread).
-// Measured on the 256^2 sweep (14.7-15.2 ms): 128-thread blocks 15.6 ms,
-// 64-thread 16.3 ms, 128 threads with the collision pass held to 85
-// registers 15.5 ms (at 1024^2 that one is 8.5 % faster, 11.6 against
-// 12.7 ms for 40 steps).
-constexpr int kRevThreads = 256;
-// The collision pass is compiled for three blocks per SM (80 registers, 8
-// bytes spilled; 96 at two): 1024^2 sweep 129.2 -> 119.9 ms, 256^2 13.83 ->
-// 13.73 ms.
+inline int rev_blocks(const StepParams &P) { return ((P.nx + kRevX - 1) / kRevX) * ((P.ny + kRevY - 1) / kRevY); }
 
-// The four reverse passes, one launch each (every pass reads what the one
-// before wrote at the neighbours).
-template <int NS>
-__global__ void __launch_bounds__(kRevThreads, 3) rev_collide_kernel(const StepParams P, AdjTape T, AdjFields A)
+// Adds the block's sums of K per-thread values to gacc[q][block] in FP64, in
+// a fixed order: thread lane l of a warp sums the values of threads l, l + 32,
+// ..., then the lanes are added pairwise.  (Per-node FP64 sums, read and
+// written every step, cost 16 bytes a node and value; FP64 additions are few
+// per SM, so the values meet in shared memory first.)
+template <int K>
+__device__ __forceinline__ void block_sums(const float (&v)[K], float *s_v, double *gacc, int first)
 {
+#pragma unroll
+    for (int q = 0; q < K; ++q) s_v[q * kRevThreads + threadIdx.x] = v[q];
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    for (int q = threadIdx.x >> 5; q < K; q += kRevThreads / 32) {
+        double a = (double)s_v[q * kRevThreads + lane];
+#pragma unroll
+        for (int w = 1; w < kRevThreads / 32; ++w) a += (double)s_v[q * kRevThreads + 32 * w + lane];
+        for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
+        if (lane == 0) gacc[(size_t)(first + q) * gridDim.x + blockIdx.x] += a;
+    }
+}
+
+template <int NS, bool GATHER, bool WALLS>
+__global__ void __launch_bounds__(kRevThreads, NS <= 2 ? 3 : (NS <= 4 ? 2 : 1)) rev_collide_kernel(const StepParams P, AdjTape T, AdjFields A)
+{
+    constexpr int K = (NS + 1) * NS / 2 + 1;
+    __shared__ float s_v[K * kRevThreads];
     pdl_wait();   // the previous kernel of the sweep has completed
-    for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < P.plane; k += gridDim.x * blockDim.x)
-        rev_collide_node<NS>(P, T, A, k);
+    const int bx = (P.nx + kRevX - 1) / kRevX, by = blockIdx.x / bx;
+    const int x = (blockIdx.x - by * bx) * kRevX + threadIdx.x % kRevX, y = by * kRevY + threadIdx.x / kRevX;
+    float sums[K];
+#pragma unroll
+    for (int q = 0; q < K; ++q) sums[q] = 0.f;
+    if (x < P.nx && y < P.ny) rev_collide_node<NS, GATHER, WALLS>(P, T, A, x, y, (unsigned)y * P.nx + x, sums);
+    block_sums<K>(sums, s_v, A.gacc, 0);
 }
 
+// rev2 and rev3 on a tile.  rev2 runs on the tile and, for what rev3 gathers,
+// on a one-node ring around it (a third of it twice, from lines that are in
+// L2); its gradient adjoints stay in shared memory.  rev3: the gradient and
+// Laplacian stencils transposed: phi_p(z) entered grad phi_p(z - c_i) with
+// weight 3 w_i c_i and lap phi_p(z - c_i) with 6 w_i (and lap phi_p(z) with
+// -6 (1 - w_0)).
 template <int NS, int MODEL, bool WALLS>
-__global__ void rev_source_kernel(const StepParams P, AdjTape T, AdjFields A)
+__global__ void __launch_bounds__(kRevThreads) rev_source_kernel(const StepParams P, AdjTape T, AdjFields A)
 {
+    constexpr int RX = kRevX + 2, RN = RX * (kRevY + 2);
+    __shared__ float s_l[3 * NS * RN];   // per phase: x and y gradient adjoints, Laplacian adjoint
+    __shared__ float s_v[kRevThreads];
     pdl_wait();
-    for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < P.plane; k += gridDim.x * blockDim.x)
-        rev_source_node<NS, MODEL, WALLS>(P, T, A, k);
+    const unsigned pl = P.plane;
+    const int bx = (P.nx + kRevX - 1) / kRevX, by = blockIdx.x / bx;
+    const int x0 = (blockIdx.x - by * bx) * kRevX, y0 = by * kRevY;
+    const int t = threadIdx.x, lx = t % kRevX, ly = t / kRevX, x = x0 + lx, y = y0 + ly;
+    const int We = min(kRevX, P.nx - x0), He = min(kRevY, P.ny - y0);
+    const bool own = lx < We && ly < He;
+    const unsigned k = (unsigned)y * P.nx + x;
+    auto put = [&](int r, unsigned n, const float (&gx)[NS], const float (&gy)[NS]) {
+#pragma unroll
+        for (int p = 0; p < NS; ++p) {
+            s_l[(3 * p) * RN + r] = gx[p];
+            s_l[(3 * p + 1) * RN + r] = gy[p];
+            s_l[(3 * p + 2) * RN + r] = __ldg(A.llap + (size_t)p * pl + n);
+        }
+    };
+    float pw[NS], sums[1] = {0.f};
+    if (own) {
+        float d_ph[NS], gx[NS], gy[NS], d_ux, d_uy;
+        rev_source_node<NS, MODEL, WALLS>(P, T, A, x, y, k, d_ph, gx, gy, d_ux, d_uy, sums[0]);
+        const float lux = A.lu_in[k], luy = A.lu_in[pl + k];
+#pragma unroll
+        for (int p = 0; p < NS; ++p) pw[p] = __ldg(A.lphi_pw + (size_t)p * pl + k) + d_ph[p];
+        put((ly + 1) * RX + lx + 1, k, gx, gy);
+        A.lu_in[k] = lux + d_ux;
+        A.lu_in[pl + k] = luy + d_uy;
+    }
+    for (int h = t; h < 2 * RX + 2 * kRevY; h += kRevThreads) {
+        int rx, ry;   // offset from (x0, y0)
+        if (h < 2 * RX) {
+            const int r = h >= RX;
+            rx = h - r * RX - 1;
+            ry = r ? He : -1;
+        } else {
+            const int q = h - 2 * RX;
+            ry = q >> 1;
+            rx = (q & 1) ? We : -1;
+        }
+        if (rx > We || (h >= 2 * RX && ry >= He) || (WALLS && beyond_wall(P, x0 + rx, y0 + ry))) continue;
+        const unsigned n = wrap_node(x0 + rx, y0 + ry, P.nx, P.ny);
+        float d_ph[NS], gx[NS], gy[NS], a, b, c;
+        rev_source_node<NS, MODEL, WALLS>(P, T, A, (int)(n % (unsigned)P.nx), (int)(n / (unsigned)P.nx), n, d_ph, gx, gy, a,
+                                          b, c);
+        put((ry + 1) * RX + rx + 1, n, gx, gy);
+    }
+    block_sums<1>(sums, s_v, A.gacc, (NS + 1) * NS / 2);   // its barrier also closes s_l
+    if (own) {
+        const int c = (ly + 1) * RX + lx + 1;
+#pragma unroll
+        for (int p = 0; p < NS; ++p) {
+            const float *lgx = s_l + (3 * p) * RN + c, *lgy = lgx + RN, *ll = lgy + RN;
+            float a = pw[p] - 6.f * (1.f - 4.f / 9.f) * ll[0];
+            if constexpr (!WALLS) {
+#pragma unroll
+                for (int i = 1; i < 9; ++i) {
+                    const int n = -cyi(i) * RX - cxi(i);
+                    float g = cxi(i) != 0 ? (cxi(i) > 0 ? lgx[n] : -lgx[n]) : 0.f;
+                    if (cyi(i) != 0) g += cyi(i) > 0 ? lgy[n] : -lgy[n];
+                    a += 3.f * wgt(i) * g + 6.f * wgt(i) * ll[n];
+                }
+            } else {
+                // phi of this node also stands at its ghosts beyond the walls
+                int px[9], py[9];
+                const int ns = standins(P, x, y, px, py);
+                for (int s = 0; s < ns; ++s)
+#pragma unroll
+                    for (int i = 1; i < 9; ++i) {
+                        const int zx = px[s] - cxi(i), zy = py[s] - cyi(i);
+                        if (beyond_wall(P, zx, zy)) continue;
+                        const int n = (zy - y) * RX + zx - x;
+                        a += 3.f * wgt(i) * (cxi(i) * lgx[n] + cyi(i) * lgy[n]) + 6.f * wgt(i) * ll[n];
+                    }
+            }
+            A.lphi_tot[(size_t)p * pl + k] = a;
+        }
+    }
 }
 
 template <int NS, bool WALLS>
-__global__ void rev_stencil_kernel(const StepParams P, AdjFields A)
-{
-    pdl_wait();
-    for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < P.plane; k += gridDim.x * blockDim.x)
-        rev_stencil_node<NS, WALLS>(P, A, k);
-}
-
-template <int NS, bool WALLS>
-__global__ void rev_pull_kernel(const StepParams P, AdjFields A)
+__global__ void __launch_bounds__(256) rev_pull_kernel(const StepParams P, AdjFields A)
 {
     pdl_wait();
     for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < P.plane; k += gridDim.x * blockDim.x)
@@ -935,36 +1027,31 @@ int blocks_for(unsigned n)
 }
 
 
+template <int NS, int MODEL, bool WALLS>
+cudaError_t reverse_passes(const StepParams &P, const AdjTape &T, const AdjFields &A, bool taped, cudaStream_t st)
+{
+    const int nb = rev_blocks(P);
+    cudaError_t e = taped ? launch_pdl(rev_collide_kernel<NS, true, WALLS>, nb, kRevThreads, 0, st, P, T, A)
+                          : launch_pdl(rev_collide_kernel<NS, false, WALLS>, nb, kRevThreads, 0, st, P, T, A);
+    if (e != cudaSuccess) return e;
+    e = launch_pdl(rev_source_kernel<NS, MODEL, WALLS>, nb, kRevThreads, 0, st, P, T, A);
+    if (e != cudaSuccess || taped) return e;
+    return launch_pdl(rev_pull_kernel<NS, WALLS>, blocks_for(P.plane), 256, 0, st, P, A);
+}
+
 template <int NS, int MODEL>
 cudaError_t reverse_step_ns(const StepParams &P, const AdjTape &T, const AdjFields &A, bool taped, cudaStream_t st)
 {
     const int nb = blocks_for(P.plane);
-    const int nr = (int)((P.plane + kRevThreads - 1) / kRevThreads);
     if (!taped) {
         tape_pull_kernel<NS><<<nb, 256, 0, st>>>(P, T);
         tape_stencil_kernel<NS, MODEL><<<nb, 256, 0, st>>>(P, T);
         tape_force_kernel<NS><<<nb, 256, 0, st>>>(P, T);
     }
-    // the four passes overlap each launch with the drain of the one before
-    // (measured: one cooperative launch with grid barriers between the
-    // passes is slower, 17.2 against 14.8 ms for the 256^2 sweep; passes 2-4
-    // as one launch over tiles of 32 x 8 nodes, pass 2 recomputed on a
-    // margin of two and pass 3 on a margin of one in shared memory, give
-    // 13.42 against 13.70 ms at 256^2 but 141.9 against 128.9 ms at 1024^2,
-    // and 32 x 16, 64 x 8, 32 x 32 tiles are slower at 1024^2 as well)
-    cudaError_t e;
-    if ((e = launch_pdl(rev_collide_kernel<NS>, nr, kRevThreads, 0, st, P, T, A)) != cudaSuccess) return e;
     // periodic lattices take passes without the wall branches (fewer
     // registers, no local arrays)
-    if (P.wall_x || P.wall_y) {
-        if ((e = launch_pdl(rev_source_kernel<NS, MODEL, true>, nr, kRevThreads, 0, st, P, T, A)) != cudaSuccess)
-            return e;
-        if ((e = launch_pdl(rev_stencil_kernel<NS, true>, nr, kRevThreads, 0, st, P, A)) != cudaSuccess) return e;
-        return launch_pdl(rev_pull_kernel<NS, true>, nr, kRevThreads, 0, st, P, A);
-    }
-    if ((e = launch_pdl(rev_source_kernel<NS, MODEL, false>, nr, kRevThreads, 0, st, P, T, A)) != cudaSuccess) return e;
-    if ((e = launch_pdl(rev_stencil_kernel<NS, false>, nr, kRevThreads, 0, st, P, A)) != cudaSuccess) return e;
-    return launch_pdl(rev_pull_kernel<NS, false>, nr, kRevThreads, 0, st, P, A);
+    return P.wall_x || P.wall_y ? reverse_passes<NS, MODEL, true>(P, T, A, taped, st)
+                                : reverse_passes<NS, MODEL, false>(P, T, A, taped, st);
 }
 
 // dL/dphi_p for the solved phases from dL/dphi over all N phases (phi_N = 1 - sum).
@@ -994,6 +1081,8 @@ cudaError_t launch_reverse_step(int ns, const StepParams &P, const AdjTape &T, c
     default: return cudaErrorInvalidValue;
     }
 }
+
+int adj_sum_blocks(const StepParams &P) { return rev_blocks(P); }
 
 cudaError_t launch_grad_reduce(const double *gacc, int K, unsigned plane, double *partials, double *acc,
                                cudaStream_t st)

@@ -39,20 +39,27 @@ struct AdjFields {
     float *lR;       // [2(N-1)]
     float *lmphi;    // [2]
     float *lg_pull;  // [8]
-    float *lphi_tot; // [N-1]
-    double *gacc;    // [N(N-1)/2 + 1] per-node sums over the steps of dL/dsigma_pq
-                     // (pair order p<q) and dL/dM, FP64
+    float *lphi_tot; // [N-1] read at the neighbours by the next reversed step's first pass
+    // the sweep's first pass: lj and lg_pull of the step reversed before (the
+    // following step), while it writes this step's
+    const float *lj_next, *lg_next;
+    double *gacc;    // [N(N-1)/2 + 1][adj_sum_blocks] sums over the steps and a block's
+                     // nodes of dL/dsigma_pq (pair order p<q) and dL/dM, FP64
 };
 
 // Tape and reverse of one step whose input state P describes (P.fin, P.gin,
 // P.phi_prev, P.uin, P.mphi); adds this step's parameter-gradient terms to
-// A.gacc node by node.  taped: T already holds the step's intermediate
-// fields (written by the taping forward kernel), so only the four reverse
-// passes run.
+// A.gacc.  taped (a sweep): T already holds the step's intermediate fields
+// (written by the taping forward kernel), the seeds of the populations are
+// gathered from lphi_tot, lj_next and lg_next, and lf_in, lg_in are not
+// formed: two passes.  Otherwise the tape is rebuilt, lf_out and lg_out are
+// the seeds, and a last pass writes lf_in and lg_in.
 cudaError_t launch_reverse_step(int ns, const StepParams &P, const AdjTape &T, const AdjFields &A, bool taped,
                                 cudaStream_t st);
-// acc[c] = sum over nodes of gacc[c][node], c < K, in a fixed order (FP64).
-cudaError_t launch_grad_reduce(const double *gacc, int K, unsigned plane, double *partials, double *acc,
+// Number of partial sums per parameter in gacc.
+int adj_sum_blocks(const StepParams &P);
+// acc[c] = sum of gacc[c][n] over n, c < K, in a fixed order (FP64).
+cudaError_t launch_grad_reduce(const double *gacc, int K, unsigned n, double *partials, double *acc,
                                cudaStream_t st);
 // lphi[p] = seed[p] - seed[N-1] for the N-1 solved phases.
 cudaError_t launch_fold_seed(int ns, const float *seed, unsigned plane, float *lphi, cudaStream_t st);

@@ -1233,8 +1233,8 @@ AdjTape adj_tape(const nlbm_adjoint *a, int k)
 int64_t adj_sweep_launches(const nlbm_adjoint *a)
 {
     // fold + per step: one taping step kernel while the segment is rebuilt
-    // and 4 reverse kernels; the phi0 sum and the two-kernel reduction
-    return 1 + 5 * (int64_t)a->nsteps + 1 + 2;
+    // and 2 reverse kernels; the phi0 sum and the two-kernel reduction
+    return 1 + 3 * (int64_t)a->nsteps + 1 + 2;
 }
 
 // The reverse sweep, asynchronous and capturable: seeds from seed_buf,
@@ -1248,6 +1248,8 @@ cudaError_t adj_backward_body(nlbm_adjoint *a)
     for (int k = 0; k < 2; ++k)
         if ((e = cudaMemsetAsync(a->seed[k], 0, pb * c.seedset, a->stream)) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(a->A.gacc, 0, pb * c.contrib, a->stream)) != cudaSuccess) return e;
+    // no step follows the last: what its first pass gathers is 0
+    if ((e = cudaMemsetAsync(a->A.lphi_tot, 0, pb * ns, a->stream)) != cudaSuccess) return e;
     if ((e = launch_fold_seed(ns, a->seed_buf, (unsigned)pl, a->seed[0] + pl * (9 * ns + 8), a->stream)) != cudaSuccess)
         return e;
     int cur = 0;
@@ -1277,7 +1279,13 @@ cudaError_t adj_backward_body(nlbm_adjoint *a)
         }
         for (int s = len - 1; s >= 0; --s) {
             const StepParams kp = adj_params_from_state(a, a->seg + a->state_floats * s);
-            const AdjFields A = adj_fields(a, a->seed[cur], a->seed[cur ^ 1]);
+            AdjFields A = adj_fields(a, a->seed[cur], a->seed[cur ^ 1]);
+            // the sweep's seed sets hold j and pulled g adjoints (2 ns + 8
+            // planes) where a single step's hold those of the populations
+            A.lj_next = a->seed[cur];
+            A.lg_next = a->seed[cur] + 2 * ns * pl;
+            A.lj = a->seed[cur ^ 1];
+            A.lg_pull = a->seed[cur ^ 1] + 2 * ns * pl;
             if ((e = launch_reverse_step(ns, kp, adj_tape(a, s), A, true, a->stream)) != cudaSuccess) return e;
             cur ^= 1;
         }
@@ -1289,7 +1297,7 @@ cudaError_t adj_backward_body(nlbm_adjoint *a)
     if ((e = launch_add_planes(a->A.lphi_tot, lphi_in, (unsigned)(pl * ns), a->grad_buf, a->stream)) != cudaSuccess)
         return e;
     const int np = (ns + 1) * ns / 2;
-    return launch_grad_reduce(a->A.gacc, np + 1, (unsigned)pl, a->partials, a->acc, a->stream);
+    return launch_grad_reduce(a->A.gacc, np + 1, (unsigned)adj_sum_blocks(a->sim->kp), a->partials, a->acc, a->stream);
 }
 
 }  // namespace
@@ -1471,9 +1479,9 @@ nlbm_status nlbm_adjoint_reverse_step(nlbm_adjoint *a, const float *dev_state, c
         return adj_fail(a, e, "seed");
     const StepParams kp = adj_params_from_state(a, dev_state);
     if ((e = launch_reverse_step(ns, kp, a->T, adj_fields(a, a->seed[0], a->seed[1]), false, a->stream)) != cudaSuccess ||
-        (e = launch_grad_reduce(a->A.gacc, np + 1, (unsigned)pl, a->partials, a->acc, a->stream)) != cudaSuccess)
+        (e = launch_grad_reduce(a->A.gacc, np + 1, (unsigned)adj_sum_blocks(kp), a->partials, a->acc, a->stream)) != cudaSuccess)
         return adj_fail(a, e, "reverse step");
-    a->sim->launches += 9;
+    a->sim->launches += 8;
     double acc[kMaxPhases * kMaxPhases + 1];
     if ((e = cudaMemcpyAsync(dev_seed_in, a->seed[1], pb * c.seedset, cudaMemcpyDeviceToDevice, a->stream)) != cudaSuccess ||
         (e = cudaMemcpyAsync(acc, a->acc, sizeof(double) * (np + 1), cudaMemcpyDeviceToHost, a->stream)) != cudaSuccess ||
