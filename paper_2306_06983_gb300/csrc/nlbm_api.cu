@@ -1087,7 +1087,7 @@ struct nlbm_adjoint {
     double *partials, *acc;    // [kAdjRedBlocks][NP+1], [NP+1]
     float *seed_buf;           // [N][plane] copy of the caller's dL/dphi(T)
     float *grad_buf;           // [N-1][plane] dL/dphi_0
-    int final_set;             // seed set holding step 1's input adjoints
+    int taped;                 // segment whose states and tapes seg / tapes hold, -1: none
     cudaGraphExec_t graph;     // the whole reverse sweep, captured on first use
     bool graph_tried;
     bool forward_done;
@@ -1159,23 +1159,6 @@ nlbm_status adj_fail(nlbm_adjoint *a, cudaError_t e, const char *what)
     return NLBM_ECUDA;
 }
 
-// Copy the simulation's current state into / out of a packed state record.
-cudaError_t adj_save_state(nlbm_adjoint *a, float *dst)
-{
-    nlbm_sim *s = a->sim;
-    const size_t pl = a->plane, pb = sizeof(float) * pl;
-    const int c = s->cur;
-    struct Part { const void *src; size_t n; } parts[] = {
-        {s->f(c), pb * 9 * a->ns}, {s->g(c), pb * 8}, {s->u(c), pb * 2}, {s->phi(c), pb * a->ns}, {s->mphi(), pb * 2}};
-    char *d = (char *)dst;
-    for (const Part &p : parts) {
-        cudaError_t e = cudaMemcpyAsync(d, p.src, p.n, cudaMemcpyDeviceToDevice, a->stream);
-        if (e != cudaSuccess) return e;
-        d += p.n;
-    }
-    return cudaSuccess;
-}
-
 // Step parameters whose inputs are a packed state record.
 StepParams adj_params_from_state(const nlbm_adjoint *a, const float *state)
 {
@@ -1188,6 +1171,50 @@ StepParams adj_params_from_state(const nlbm_adjoint *a, const float *state)
     kp.mphi = const_cast<float *>(kp.phi_prev + pl * a->ns);
     kp.mphi_in = kp.mphi;
     return kp;
+}
+
+// One forward step from one packed state record to another; tape: also the
+// step's intermediate fields.
+cudaError_t adj_step(nlbm_adjoint *a, const float *in, float *out, float *tape)
+{
+    const size_t pl = a->plane;
+    const int ns = a->ns;
+    StepParams kp = adj_params_from_state(a, in);
+    kp.fout = out;
+    kp.gout = out + pl * 9 * ns;
+    kp.uout = kp.gout + pl * 8;
+    kp.phi = kp.uout + pl * 2;
+    kp.mphi = kp.phi + pl * ns;   // read from the input state, written to the output
+    kp.pout = nullptr;
+    kp.tape = tape;
+    if (!tape) return launch_step(a->sim, kp);
+    return (kp.model == NLBM_MODEL_A ? launch_step_tape_a_f32 : launch_step_tape_b_f32)(ns, kp, a->stream);
+}
+
+// Input state of step s (0-based) of segment k: the checkpoint, then the
+// states that the segment's own steps wrote.
+float *adj_segment_state(const nlbm_adjoint *a, int k, int s)
+{
+    return s == 0 ? a->ckpt + a->state_floats * k : a->seg + a->state_floats * s;
+}
+
+int adj_segment_length(const nlbm_adjoint *a, int k)
+{
+    return (k + 1) * a->every <= a->nsteps ? a->every : a->nsteps - k * a->every;
+}
+
+// The states and tapes of segment k from its checkpoint: one taping step
+// launch per step (the last step's output state goes to the spare slot).
+cudaError_t adj_tape_segment(nlbm_adjoint *a, int k)
+{
+    const size_t tape = a->plane * (size_t)adj_counts(a->ns).tape;
+    const int len = adj_segment_length(a, k);
+    for (int s = 0; s < len; ++s) {
+        const cudaError_t e =
+            adj_step(a, adj_segment_state(a, k, s), a->seg + a->state_floats * (s + 1), a->tapes + tape * s);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 // Adjoint-field pointers for a step whose output adjoints are seed set so
@@ -1230,55 +1257,36 @@ AdjTape adj_tape(const nlbm_adjoint *a, int k)
 }
 
 // Kernel launches of one reverse sweep (counted, not queried).
-int64_t adj_sweep_launches(const nlbm_adjoint *a)
+int64_t adj_sweep_launches(const nlbm_adjoint *a, bool rebuild_last)
 {
-    // fold + per step: one taping step kernel while the segment is rebuilt
-    // and 2 reverse kernels; the phi0 sum and the two-kernel reduction
-    return 1 + 3 * (int64_t)a->nsteps + 1 + 2;
+    // fold + per step: 2 reverse kernels and, unless forward has kept the
+    // last segment's tapes, one taping step kernel while its segment is
+    // rebuilt; the phi0 sum and the two-kernel reduction
+    const int64_t kept = rebuild_last ? 0 : adj_segment_length(a, a->nckpt - 1);
+    return 1 + 3 * (int64_t)a->nsteps - kept + 1 + 2;
 }
 
 // The reverse sweep, asynchronous and capturable: seeds from seed_buf,
 // dL/dphi_0 into grad_buf, dL/dsigma and dL/dM into acc.
-cudaError_t adj_backward_body(nlbm_adjoint *a)
+cudaError_t adj_backward_body(nlbm_adjoint *a, bool rebuild_last)
 {
     const size_t pl = a->plane, pb = sizeof(float) * pl;
-    const int ns = a->ns;
-    const AdjCounts c = adj_counts(ns);
+    const int ns = a->ns, np = (ns + 1) * ns / 2, blocks = adj_sum_blocks(a->sim->kp);
     cudaError_t e;
-    for (int k = 0; k < 2; ++k)
-        if ((e = cudaMemsetAsync(a->seed[k], 0, pb * c.seedset, a->stream)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(a->A.gacc, 0, pb * c.contrib, a->stream)) != cudaSuccess) return e;
-    // no step follows the last: what its first pass gathers is 0
+    // No step follows the last: what its first pass gathers (the adjoints of
+    // j and of the pulled g in the seed set, of phi in lphi_tot) is 0, and so
+    // are the seeds of u and m_phi.
+    if ((e = cudaMemsetAsync(a->seed[0], 0, pb * (2 * ns + 8), a->stream)) != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(a->seed[0] + pl * (10 * ns + 8), 0, pb * 4, a->stream)) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(a->A.lphi_tot, 0, pb * ns, a->stream)) != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(a->A.gacc, 0, sizeof(double) * (np + 1) * blocks, a->stream)) != cudaSuccess) return e;
     if ((e = launch_fold_seed(ns, a->seed_buf, (unsigned)pl, a->seed[0] + pl * (9 * ns + 8), a->stream)) != cudaSuccess)
         return e;
     int cur = 0;
     for (int k = a->nckpt - 1; k >= 0; --k) {
-        const int t0 = k * a->every;
-        const int len = (k + 1) * a->every <= a->nsteps ? a->every : a->nsteps - t0;
-        // rebuild the segment's input states S_t0 .. S_t0+len-1 in place and,
-        // with the same launches, the tape of each of its steps (the last
-        // step's output state goes to the spare slot)
-        if ((e = cudaMemcpyAsync(a->seg, a->ckpt + a->state_floats * k, sizeof(float) * a->state_floats,
-                                 cudaMemcpyDeviceToDevice, a->stream)) != cudaSuccess)
-            return e;
-        for (int s = 1; s <= len; ++s) {
-            const float *in = a->seg + a->state_floats * (s - 1);
-            float *out = a->seg + a->state_floats * s;
-            StepParams kp = adj_params_from_state(a, in);
-            kp.fout = out;
-            kp.gout = out + pl * 9 * ns;
-            kp.uout = kp.gout + pl * 8;
-            kp.phi = kp.uout + pl * 2;
-            kp.mphi = kp.phi + pl * ns;   // read from the input state, written to the output
-            kp.pout = nullptr;
-            kp.tape = a->tapes + pl * (size_t)c.tape * (s - 1);
-            if ((e = (kp.model == NLBM_MODEL_A ? launch_step_tape_a_f32 : launch_step_tape_b_f32)(ns, kp, a->stream)) !=
-                cudaSuccess)
-                return e;
-        }
-        for (int s = len - 1; s >= 0; --s) {
-            const StepParams kp = adj_params_from_state(a, a->seg + a->state_floats * s);
+        if ((k < a->nckpt - 1 || rebuild_last) && (e = adj_tape_segment(a, k)) != cudaSuccess) return e;
+        for (int s = adj_segment_length(a, k) - 1; s >= 0; --s) {
+            const StepParams kp = adj_params_from_state(a, adj_segment_state(a, k, s));
             AdjFields A = adj_fields(a, a->seed[cur], a->seed[cur ^ 1]);
             // the sweep's seed sets hold j and pulled g adjoints (2 ns + 8
             // planes) where a single step's hold those of the populations
@@ -1290,14 +1298,12 @@ cudaError_t adj_backward_body(nlbm_adjoint *a)
             cur ^= 1;
         }
     }
-    a->final_set = cur;
     // phi0 entered step 1 as its pulled phase populations (f_i = w_i phi0,
     // so the adjoint is that of phi) and as its phi_prev
     const float *lphi_in = a->seed[cur] + pl * (9 * ns + 8);
     if ((e = launch_add_planes(a->A.lphi_tot, lphi_in, (unsigned)(pl * ns), a->grad_buf, a->stream)) != cudaSuccess)
         return e;
-    const int np = (ns + 1) * ns / 2;
-    return launch_grad_reduce(a->A.gacc, np + 1, (unsigned)adj_sum_blocks(a->sim->kp), a->partials, a->acc, a->stream);
+    return launch_grad_reduce(a->A.gacc, np + 1, (unsigned)blocks, a->partials, a->acc, a->stream);
 }
 
 }  // namespace
@@ -1386,7 +1392,7 @@ nlbm_status nlbm_adjoint_create(const nlbm_params *p, int32_t nsteps, int32_t ch
     a->grad_buf = take(ns);
     a->partials = (double *)(ws + L.partials);
     a->acc = (double *)(ws + L.acc);
-    a->final_set = 0;
+    a->taped = -1;
     a->graph = nullptr;
     a->graph_tried = false;
     a->forward_done = false;
@@ -1402,15 +1408,40 @@ nlbm_status nlbm_adjoint_forward(nlbm_adjoint *a, const float *dev_phi0, float *
     s->cur = 0;
     nlbm_status st = nlbm_set_phi(s, dev_phi0);
     if (st != NLBM_OK) { memcpy(a->err, s->err, sizeof a->err); return st; }
+    // The initial state becomes the first checkpoint; from there on a step
+    // reads one packed record and writes the next, every segment's last step
+    // straight into the next checkpoint.  The last segment runs the taping
+    // kernel: its states and tapes are the first that a sweep needs.
+    const size_t pl = a->plane, pb = sizeof(float) * pl;
+    const int c = s->cur, ns = a->ns, last = a->nckpt - 1;
+    struct Part { const void *src; size_t n; } parts[] = {
+        {s->f(c), pb * 9 * ns}, {s->g(c), pb * 8}, {s->u(c), pb * 2}, {s->phi(c), pb * ns}, {s->mphi(), pb * 2}};
     cudaError_t e;
-    for (int k = 0; k < a->nckpt; ++k) {
-        if ((e = adj_save_state(a, a->ckpt + a->state_floats * k)) != cudaSuccess) return adj_fail(a, e, "checkpoint");
-        const int n = (k + 1) * a->every <= a->nsteps ? a->every : a->nsteps - k * a->every;
-        if ((st = nlbm_step(s, n)) != NLBM_OK) { memcpy(a->err, s->err, sizeof a->err); return st; }
+    char *d = (char *)a->ckpt;
+    for (const Part &p : parts) {
+        if ((e = cudaMemcpyAsync(d, p.src, p.n, cudaMemcpyDeviceToDevice, a->stream)) != cudaSuccess)
+            return adj_fail(a, e, "checkpoint");
+        d += p.n;
     }
-    if (dev_phi_final && (st = nlbm_get_moments(s, dev_phi_final, nullptr, nullptr)) != NLBM_OK) {
-        memcpy(a->err, s->err, sizeof a->err);
-        return st;
+    a->forward_done = false;
+    a->taped = -1;
+    for (int k = 0; k < last; ++k) {
+        const float *in = a->ckpt + a->state_floats * k;
+        for (int t = 0; t < a->every; ++t) {
+            float *out = t + 1 < a->every ? a->seg + a->state_floats * (t & 1) : a->ckpt + a->state_floats * (k + 1);
+            if ((e = adj_step(a, in, out, nullptr)) != cudaSuccess) return adj_fail(a, e, "forward step");
+            in = out;
+        }
+    }
+    if ((e = adj_tape_segment(a, last)) != cudaSuccess) return adj_fail(a, e, "forward step");
+    s->launches += a->nsteps;
+    a->taped = last;
+    if (dev_phi_final) {
+        const float *end = a->seg + a->state_floats * adj_segment_length(a, last);
+        e = launch_export(ns, end + pl * (9 * ns + 10), nullptr, nullptr, (unsigned)pl, dev_phi_final, nullptr, nullptr,
+                          a->stream);
+        if (e != cudaSuccess) return adj_fail(a, e, "export kernel");
+        s->launches++;
     }
     a->forward_done = true;
     return NLBM_OK;
@@ -1426,14 +1457,16 @@ nlbm_status nlbm_adjoint_backward(nlbm_adjoint *a, const float *dev_seed, float 
     const AdjCounts c = adj_counts(ns);
     cudaError_t e = cudaMemcpyAsync(a->seed_buf, dev_seed, pb * N, cudaMemcpyDeviceToDevice, a->stream);
     if (e != cudaSuccess) return adj_fail(a, e, "seed copy");
-    // The sweep is the same sequence of launches for every call of this
-    // handle: capture it into a CUDA graph once (on a capturable stream) and
-    // replay it.
-    if (!a->graph && !a->graph_tried && a->stream != nullptr) {
+    // After a forward the sweep is the same sequence of launches on every
+    // call of this handle: capture it into a CUDA graph once (on a capturable
+    // stream) and replay it.  A second sweep after one forward has to rebuild
+    // the last segment too.
+    const bool rebuild_last = a->taped != a->nckpt - 1;
+    if (!rebuild_last && !a->graph && !a->graph_tried && a->stream != nullptr) {
         a->graph_tried = true;
         cudaGraph_t g = nullptr;
         if (cudaStreamBeginCapture(a->stream, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
-            cudaError_t eb = adj_backward_body(a);
+            cudaError_t eb = adj_backward_body(a, false);
             cudaError_t ec = cudaStreamEndCapture(a->stream, &g);
             if (eb == cudaSuccess && ec == cudaSuccess && cudaGraphInstantiate(&a->graph, g, 0) != cudaSuccess)
                 a->graph = nullptr;
@@ -1441,13 +1474,14 @@ nlbm_status nlbm_adjoint_backward(nlbm_adjoint *a, const float *dev_seed, float 
         }
         cudaGetLastError();   // a failed capture leaves the direct path
     }
-    if (a->graph) {
+    a->taped = 0;   // the segment that the sweep ends with
+    if (a->graph && !rebuild_last) {
         e = cudaGraphLaunch(a->graph, a->stream);
         if (e != cudaSuccess) return adj_fail(a, e, "graph launch");
-    } else if ((e = adj_backward_body(a)) != cudaSuccess) {
+    } else if ((e = adj_backward_body(a, rebuild_last)) != cudaSuccess) {
         return adj_fail(a, e, "reverse sweep");
     }
-    a->sim->launches += adj_sweep_launches(a);
+    a->sim->launches += adj_sweep_launches(a, rebuild_last);
     if (dev_grad_phi0 &&
         (e = cudaMemcpyAsync(dev_grad_phi0, a->grad_buf, pb * ns, cudaMemcpyDeviceToDevice, a->stream)) != cudaSuccess)
         return adj_fail(a, e, "phi0 gradient");
