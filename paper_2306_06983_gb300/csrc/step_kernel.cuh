@@ -1732,7 +1732,7 @@ cudaError_t launch_step_nst(const StepParams &p, int ty, cudaStream_t st)
     e = vec ? variant_slots<NS, MODEL, T, ST, true, TAPE>(dev, &slots)
             : variant_slots<NS, MODEL, T, ST, false, TAPE>(dev, &slots);
     if (e != cudaSuccess) return e;
-    if (ty <= 0 && use_patches<NS, ST>(p.ny, march_chunks(p, T, slots)))
+    if (ty <= 0 && use_patches<NS, MODEL, ST>(p.ny, march_chunks(p, T, slots), vec))
         return launch_patches<NS, MODEL, ST, TAPE>(p, st);
     return vec ? launch_step_variant<NS, MODEL, T, ST, true, TAPE>(p, ty, slots, st)
                : launch_step_variant<NS, MODEL, T, ST, false, TAPE>(p, ty, slots, st);

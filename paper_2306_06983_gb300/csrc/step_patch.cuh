@@ -261,21 +261,27 @@ cudaError_t launch_patch_variant(const StepParams &p, cudaStream_t st)
 }
 
 // Patch shapes and the blocks per SM they are compiled for.  Narrow patches
-// (16 x 8, 128 threads) put a small lattice on more SMs and need fewer
-// registers per SM for one more block in flight (N = 5, 1024^2: 98.1 us a
-// step with four blocks, 91.5 with five; N = 7: 152 with five, spilling, 146
-// with four).  Wide ones (32 x 8, 256 threads) repeat fewer pulls (1.69
-// against 1.88 per node) and win once they fill the GPU where their registers
-// still leave three or four blocks: FP32 at N <= 4 (2048^2 N = 3: 192 against
-// 221 us), 16-bit storage at N = 5 (2048^2: 331 against 345 us).  Patches of
-// 64 x 4, 16 x 16, 32 x 4, 32 x 16, 16 x 4 and 8 x 8 nodes were slower than
-// the better of the two by 1 to 60 %.
+// (16 x 8, 128 threads) put a small lattice on more SMs, and one more of
+// their blocks fits where registers are short (N = 5, 1024^2: 98.1 us a step
+// with four blocks, 91.5 with five).  Wide ones (32 x 8, 256 threads) repeat
+// fewer pulls (1.69 against 1.88 per node); they win once they fill the GPU
+// where their registers leave three or four blocks (FP32 at N <= 4, and at N =
+// 5 with Model A, whose source is lighter; 2048^2 N = 3: 192 against 221 us)
+// or where two blocks are all that either shape gets (N = 7, 8: 1024^2 N = 8
+// Model A 158 against 168 us).  Patches of 64 x 4, 16 x 16, 32 x 4, 32 x 16,
+// 16 x 4 and 8 x 8 nodes were slower than the better of the two by 1 to 60 %.
+template <int NS, int MODEL, int ST>
+constexpr bool wide_patches()
+{
+    return NS >= 6 || (ST == 0 ? NS <= 3 || (NS == 4 && MODEL == 0) : NS == 4);
+}
+
 template <int NS, int MODEL, int ST, bool TAPE>
 cudaError_t launch_patches(const StepParams &p, cudaStream_t st)
 {
-    constexpr int kNarrowMin = NS <= 3 ? 6 : (NS <= 5 ? 5 : 4), kWideMin = NS <= 2 ? 4 : 3;
+    constexpr int kNarrowMin = NS <= 3 ? 6 : (NS <= 5 ? 5 : 4), kWideMin = NS <= 2 ? 4 : (NS <= 4 ? 3 : 2);
     constexpr int kFill = 228;   // wide patches from 1.5 per SM on (256^2: equal, 300x150: 8 % slower)
-    if constexpr (ST == 0 ? NS <= 3 : NS == 4) {
+    if constexpr (wide_patches<NS, MODEL, ST>()) {
         if ((long long)((p.nx + 31) / 32) * ((p.ny + 7) / 8) >= kFill)
             return launch_patch_variant<NS, MODEL, ST, 32, 8, kWideMin, TAPE>(p, st);
     }
@@ -283,18 +289,22 @@ cudaError_t launch_patches(const StepParams &p, cudaStream_t st)
 }
 
 // Whether a step runs on patches rather than as a march of `chunks` row
-// chunks.  A march costs 6 extra rows a chunk, a patch 0.7 to 0.9 extra
-// pulls and a third of the sources per node (Model B, FP32, us a step, march
-// / patches, rows a chunk: 64^2 N = 3 6.4 / 3.5, 2 rows; 256^2 N = 5 15.7 /
-// 8.0, 2; 512^2 N = 5 32.0 / 24.8, 6, N = 8 56.4 / 52.5, 8; 1024^2 N = 5 94.2
-// / 91.5, 20, N = 7 141 / 146, 31; 2048^2 N = 5 340 / 366, 78).  N = 3 stays
-// ahead at every size (2048^2 200 / 192), and so does 16-bit storage, whose
-// marches are bound by instruction issue (2048^2 N = 5 342 / 331, N = 3 222 /
-// 185, N = 8 779 / 664).
-template <int NS, int ST>
-inline bool use_patches(int ny, int chunks)
+// chunks; windows: the march would stage row windows.  A march costs 6 extra
+// rows a chunk, a patch 0.7 to 0.9 extra pulls and a third of the sources per
+// node (FP32, us a step, march / patches, rows a chunk; Model B: 64^2 N = 3
+// 6.4 / 3.5, 2 rows; 256^2 N = 5 15.7 / 8.0, 2; 512^2 N = 5 32.0 / 24.8, 6, N =
+// 8 56.4 / 52.0, 8; 1024^2 N = 5 94.2 / 91.5, 20, N = 7 141.6 / 140.8, 31;
+// 2048^2 N = 5 340 / 366, 78, N = 8 651 / 683).  Ahead at every size: N = 3
+// (2048^2 200 / 192), Model A at N = 5 (339 / 330) and N = 8 (634 / 599, 1024^2
+// 172 / 158); 16-bit storage, whose marches are bound by instruction issue
+// (2048^2 N = 5 342 / 331, N = 3 222 / 185, N = 8 779 / 630); and, but for N =
+// 2, lattices that march without row windows (1021^2 N = 8 210 / 185, 2045^2
+// N = 3 221 / 209, N = 5 380 / 381).
+template <int NS, int MODEL, int ST>
+inline bool use_patches(int ny, int chunks, bool windows)
 {
-    return ST != 0 || NS == 2 || ny <= 24 * chunks;
+    if (ST != 0 || NS == 2 || (MODEL == 0 && (NS == 4 || NS == 7)) || (!windows && NS > 1)) return true;
+    return ny <= 24 * chunks;
 }
 
 }  // namespace nlbm

@@ -36,14 +36,14 @@ def state(p, phi0, tile):
 
 # Below, at and above the patch edges (16 and 32 columns, 8 rows), lattices
 # smaller than a patch or its ring, odd rows, walls on every axis; the larger
-# ones fill the GPU with wide patches (N <= 4).
+# ones fill the GPU with wide patches (N <= 5, 7 and 8).
 SIZES = [(1, 9, 0, 0), (3, 2, 0, 0), (15, 7, 0, 0), (16, 8, 0, 0), (17, 9, 0, 0), (33, 31, 1, 0), (4, 4, 1, 1),
          (48, 65, 0, 1), (67, 45, 1, 1), (64, 64, 0, 0), (511, 130, 0, 1), (512, 128, 0, 0)]
 
 
 @pytest.mark.parametrize("nx,ny,wall_x,wall_y", SIZES)
 @pytest.mark.parametrize("N,model,n", [(2, "B", 1.0), (3, "A", 1.5), (4, "B", 1.0), (5, "A", 1.0), (6, "B", 1.0),
-                                       (8, "A", 2.0)])
+                                       (7, "B", 1.0), (8, "A", 2.0)])
 def test_patches_equal_marches(nx, ny, wall_x, wall_y, N, model, n):
     p, phi0 = W.random_smooth(nx, ny, N, seed=nx + ny, model=model, model_a_n=n, wall_x=bool(wall_x),
                               wall_y=bool(wall_y), n_disks=4)
