@@ -297,13 +297,15 @@ cudaError_t launch_patches(const StepParams &p, cudaStream_t st)
 // 2048^2 N = 5 340 / 366, 78, N = 8 651 / 683).  Ahead at every size: N = 3
 // (2048^2 200 / 192), Model A at N = 5 (339 / 330) and N = 8 (634 / 599, 1024^2
 // 172 / 158); 16-bit storage, whose marches are bound by instruction issue
-// (2048^2 N = 5 342 / 331, N = 3 222 / 185, N = 8 779 / 630); and, but for N =
-// 2, lattices that march without row windows (1021^2 N = 8 210 / 185, 2045^2
-// N = 3 221 / 209, N = 5 380 / 381).
+// (2048^2 N = 5 342 / 331, N = 3 222 / 185, N = 8 779 / 630); and, where
+// patches are wide, lattices that march without row windows (1021^2 N = 8 210
+// / 185, 2045^2 N = 3 221 / 209, N = 8 761 / 700; narrow patches lose there at
+// size, N = 5 380 / 454).
 template <int NS, int MODEL, int ST>
 inline bool use_patches(int ny, int chunks, bool windows)
 {
-    if (ST != 0 || NS == 2 || (MODEL == 0 && (NS == 4 || NS == 7)) || (!windows && NS > 1)) return true;
+    if (ST != 0 || NS == 2 || (MODEL == 0 && (NS == 4 || NS == 7)) || (!windows && NS > 1 && wide_patches<NS, MODEL, ST>()))
+        return true;
     return ny <= 24 * chunks;
 }
 
