@@ -23,9 +23,13 @@ __device__ __forceinline__ float init_two_sum(float a, float b, float &e)
     return s;
 }
 
+// src: the initial phase fields (copied into P.phi on the way, unless they
+// are there already; never written here, so its loads need not wait for the
+// stores between them).  Writing every plane of the state is what bounds it.
 template <int NS>
-__global__ void init_kernel(const StepParams P, float *u_other)
+__global__ void init_kernel(const StepParams P, const float *src, float *u_other)
 {
+    pdl_wait();
     const unsigned pl = P.plane;
     for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < pl; k += gridDim.x * blockDim.x) {
         const int x = k % P.nx, y = k / P.nx;
@@ -33,19 +37,20 @@ __global__ void init_kernel(const StepParams P, float *u_other)
         for (int i = 0; i < 9; ++i) {
             int tx = x + kCx[i], ty = y + kCy[i];
             const bool out_x = tx < 0 || tx >= P.nx, out_y = ty < 0 || ty >= P.ny;
-            unsigned src;
+            unsigned z;
             if ((out_x && P.wall_x) || (out_y && P.wall_y)) {
-                src = k;
+                z = k;
             } else {
                 if (tx < 0) tx += P.nx;
                 if (tx >= P.nx) tx -= P.nx;
                 if (ty < 0) ty += P.ny;
                 if (ty >= P.ny) ty -= P.ny;
-                src = (unsigned)ty * P.nx + tx;
+                z = (unsigned)ty * P.nx + tx;
             }
 #pragma unroll
             for (int p = 0; p < NS; ++p) {
-                const float phi = P.phi[(size_t)p * pl + src];
+                const float phi = __ldg(src + (size_t)p * pl + z);
+                if (i == 0 && src != P.phi) P.phi[(size_t)p * pl + k] = phi;
                 const float p9 = phi * (1.f / 9.f);
                 float v;
                 if (i == 0) {
@@ -79,15 +84,17 @@ __global__ void init_kernel(const StepParams P, float *u_other)
 __device__ __forceinline__ float init_w(int i) { return i == 0 ? 4.f / 9.f : (i < 5 ? 1.f / 9.f : 1.f / 36.f); }
 
 template <int NS>
-__global__ void init16_kernel(const StepParams P, float *u_other, float *p_other)
+__global__ void init16_kernel(const StepParams P, const float *src, float *u_other, float *p_other)
 {
+    pdl_wait();
     const unsigned pl = P.plane;
     unsigned short *f16 = (unsigned short *)P.fout;
     unsigned short *g16 = (unsigned short *)P.gout;
     for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < pl; k += gridDim.x * blockDim.x) {
 #pragma unroll
         for (int p = 0; p < NS; ++p) {
-            const float phi = P.phi[(size_t)p * pl + k];
+            const float phi = __ldg(src + (size_t)p * pl + k);
+            if (src != P.phi) P.phi[(size_t)p * pl + k] = phi;
             float r[9];
 #pragma unroll
             for (int i = 1; i < 9; ++i) r[i] = __fmaf_rn(init_w(i), phi, 0.f);
@@ -116,26 +123,36 @@ __global__ void init16_kernel(const StepParams P, float *u_other, float *p_other
 }
 
 template <int NS>
-__global__ void export_kernel(const float *__restrict__ phi_aux, const float *__restrict__ u,
-                              const float *__restrict__ Pf, unsigned pl, float *phi_out,
+__global__ void export_kernel(const float *phi_aux, const float *u, const float *Pf, unsigned pl, float *phi_out,
                               float *u_out, float *p_out)
 {
+    pdl_wait();
     for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < pl; k += gridDim.x * blockDim.x) {
+        // every load before the first store
+        float ph[NS], ux = 0.f, uy = 0.f, pr = 0.f;
+        if (phi_out) {
+#pragma unroll
+            for (int p = 0; p < NS; ++p) ph[p] = phi_aux[(size_t)p * pl + k];
+        }
+        if (u_out) {
+            ux = u[k];
+            uy = u[pl + k];
+        }
+        if (p_out) pr = Pf[k];
         if (phi_out) {
             float s = 0.f;
 #pragma unroll
             for (int p = 0; p < NS; ++p) {
-                const float v = phi_aux[(size_t)p * pl + k];
-                phi_out[(size_t)p * pl + k] = v;
-                s += v;
+                phi_out[(size_t)p * pl + k] = ph[p];
+                s += ph[p];
             }
             phi_out[(size_t)NS * pl + k] = 1.f - s;   // Sec. 4: phi_N = 1 - sum
         }
         if (u_out) {
-            u_out[k] = u[k];
-            u_out[pl + k] = u[pl + k];
+            u_out[k] = ux;
+            u_out[pl + k] = uy;
         }
-        if (p_out) p_out[k] = Pf[k];
+        if (p_out) p_out[k] = pr;
     }
 }
 
@@ -223,7 +240,7 @@ int grid_for(unsigned pl, int threads)
 
 }  // namespace
 
-cudaError_t launch_init(int ns, const StepParams &p, cudaStream_t st)
+cudaError_t launch_init(int ns, const StepParams &p, const float *src, cudaStream_t st)
 {
     // p.uin is the second velocity buffer (both are zeroed).
     const int threads = 256, blocks = grid_for(p.plane, threads);
@@ -232,21 +249,19 @@ cudaError_t launch_init(int ns, const StepParams &p, cudaStream_t st)
         float *p_other = const_cast<float *>(p.pin);
         switch (ns) {
 #define NLBM_CASE(K) \
-    case K: init16_kernel<K><<<blocks, threads, 0, st>>>(p, u_other, p_other); break;
+    case K: return launch_pdl(init16_kernel<K>, dim3(blocks), dim3(threads), 0, st, p, src, u_other, p_other);
             NLBM_CASE(1) NLBM_CASE(2) NLBM_CASE(3) NLBM_CASE(4) NLBM_CASE(5) NLBM_CASE(6) NLBM_CASE(7)
 #undef NLBM_CASE
         default: return cudaErrorInvalidValue;
         }
-        return cudaGetLastError();
     }
     switch (ns) {
 #define NLBM_CASE(K) \
-    case K: init_kernel<K><<<blocks, threads, 0, st>>>(p, u_other); break;
+    case K: return launch_pdl(init_kernel<K>, dim3(blocks), dim3(threads), 0, st, p, src, u_other);
         NLBM_CASE(1) NLBM_CASE(2) NLBM_CASE(3) NLBM_CASE(4) NLBM_CASE(5) NLBM_CASE(6) NLBM_CASE(7)
 #undef NLBM_CASE
     default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 
 cudaError_t launch_export(int ns, const float *phi_aux, const float *u, const float *Pf,
@@ -255,16 +270,14 @@ cudaError_t launch_export(int ns, const float *phi_aux, const float *u, const fl
 {
     const int threads = 256, blocks = grid_for(plane, threads);
     switch (ns) {
-#define NLBM_CASE(K)                                                                          \
-    case K:                                                                                   \
-        export_kernel<K><<<blocks, threads, 0, st>>>(phi_aux, u, Pf, plane, phi_out, u_out,   \
-                                                     p_out);                                  \
-        break;
+#define NLBM_CASE(K)                                                                                              \
+    case K:                                                                                                       \
+        return launch_pdl(export_kernel<K>, dim3(blocks), dim3(threads), 0, st, phi_aux, u, Pf, plane, phi_out,   \
+                          u_out, p_out);
         NLBM_CASE(1) NLBM_CASE(2) NLBM_CASE(3) NLBM_CASE(4) NLBM_CASE(5) NLBM_CASE(6) NLBM_CASE(7)
 #undef NLBM_CASE
     default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 
 cudaError_t launch_phase_mass(int ns, const float *phi_aux, unsigned plane, double *partials,

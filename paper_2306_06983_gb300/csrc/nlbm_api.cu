@@ -245,14 +245,14 @@ StepParams step_params(const nlbm_sim *s, int a, int b)
     return kp;
 }
 
-// Initial state into the buffers of state c from the phase fields in phi(c).
-cudaError_t launch_initial_state(nlbm_sim *s, int c)
+// Initial state into the buffers of state c from the phase fields src.
+cudaError_t launch_initial_state(nlbm_sim *s, int c, const float *src)
 {
     // init writes the populations of state c; kp.uin / kp.pin name the
     // other velocity / pressure buffers, zeroed as well
     StepParams kp = step_params(s, c ^ 1, c);
     kp.phi = s->phi(c);
-    return launch_init(s->ns, kp, s->stream);
+    return launch_init(s->ns, kp, src, s->stream);
 }
 
 cudaError_t launch_step(const nlbm_sim *s, const StepParams &kp)
@@ -320,10 +320,7 @@ nlbm_status nlbm_create(const nlbm_params *p, void *dev_workspace, size_t worksp
 nlbm_status nlbm_set_phi(nlbm_sim *s, const float *dev_phi)
 {
     if (!s || !dev_phi) return NLBM_EINVAL;
-    cudaError_t e = cudaMemcpyAsync(s->phi(s->cur), dev_phi, sizeof(float) * s->ns * s->plane,
-                                    cudaMemcpyDeviceToDevice, s->stream);
-    if (e != cudaSuccess) return cuda_fail(s, e, "copy of the initial phase fields");
-    e = launch_initial_state(s, s->cur);
+    cudaError_t e = launch_initial_state(s, s->cur, dev_phi);
     if (e != cudaSuccess) return cuda_fail(s, e, "init kernel");
     s->launches++;
     s->steps = 0;
@@ -337,7 +334,7 @@ nlbm_status nlbm_set_phi_host(nlbm_sim *s, const float *host_phi)
                                     cudaMemcpyHostToDevice, s->stream);
     if (e != cudaSuccess) return cuda_fail(s, e, "upload of the initial phase fields");
     // the device copy in the phi planes is its own source for the init kernel
-    e = launch_initial_state(s, s->cur);
+    e = launch_initial_state(s, s->cur, s->phi(s->cur));
     if (e != cudaSuccess) return cuda_fail(s, e, "init kernel");
     s->launches++;
     s->steps = 0;
@@ -1405,24 +1402,22 @@ nlbm_status nlbm_adjoint_forward(nlbm_adjoint *a, const float *dev_phi0, float *
 {
     if (!a || !dev_phi0) return NLBM_EINVAL;
     nlbm_sim *s = a->sim;
-    s->cur = 0;
-    nlbm_status st = nlbm_set_phi(s, dev_phi0);
-    if (st != NLBM_OK) { memcpy(a->err, s->err, sizeof a->err); return st; }
-    // The initial state becomes the first checkpoint; from there on a step
-    // reads one packed record and writes the next, every segment's last step
-    // straight into the next checkpoint.  The last segment runs the taping
-    // kernel: its states and tapes are the first that a sweep needs.
-    const size_t pl = a->plane, pb = sizeof(float) * pl;
-    const int c = s->cur, ns = a->ns, last = a->nckpt - 1;
-    struct Part { const void *src; size_t n; } parts[] = {
-        {s->f(c), pb * 9 * ns}, {s->g(c), pb * 8}, {s->u(c), pb * 2}, {s->phi(c), pb * ns}, {s->mphi(), pb * 2}};
-    cudaError_t e;
-    char *d = (char *)a->ckpt;
-    for (const Part &p : parts) {
-        if ((e = cudaMemcpyAsync(d, p.src, p.n, cudaMemcpyDeviceToDevice, a->stream)) != cudaSuccess)
-            return adj_fail(a, e, "checkpoint");
-        d += p.n;
-    }
+    // The initial state is written as the first checkpoint; from there on a
+    // step reads one packed record and writes the next, every segment's last
+    // step straight into the next checkpoint.  The last segment runs the
+    // taping kernel: its states and tapes are the first that a sweep needs.
+    const size_t pl = a->plane;
+    const int ns = a->ns, last = a->nckpt - 1;
+    StepParams kp = adj_params_from_state(a, a->ckpt);
+    kp.fout = a->ckpt;
+    kp.gout = a->ckpt + pl * 9 * ns;
+    kp.uout = kp.gout + pl * 8;
+    kp.uin = kp.uout;             // one velocity buffer in a record
+    kp.phi = kp.uout + pl * 2;
+    kp.pout = s->P(0);
+    cudaError_t e = launch_init(ns, kp, dev_phi0, a->stream);
+    if (e != cudaSuccess) return adj_fail(a, e, "initial state");
+    s->launches++;
     a->forward_done = false;
     a->taped = -1;
     for (int k = 0; k < last; ++k) {

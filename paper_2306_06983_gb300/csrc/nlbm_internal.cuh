@@ -75,8 +75,8 @@ struct StepParams {
     float wetc[2][kMaxPhases][kMaxPhases];   // (4/eps) cos theta_pq, walls y = 0 and y = ny - 1
 };
 
-// Programmatic dependent launch (the step kernels, the ensemble kernel and the
-// adjoint's reverse passes): a kernel launched with launch_pdl is scheduled
+// Programmatic dependent launch (the step kernels, the ensemble kernels, the
+// adjoint's reverse passes, the initial state and the export): a kernel launched with launch_pdl is scheduled
 // as the blocks of its
 // predecessor in the stream exit, so its launch overlaps their drain.  It
 // must call pdl_wait() before touching memory the predecessor reads or
@@ -142,7 +142,8 @@ cudaError_t launch_batch_patches(int ns, int px, const StepParams *d_params, con
                                  int *d_counters, int parity, cudaStream_t st);
 
 // Auxiliary kernels (aux_kernels.cu).
-cudaError_t launch_init(int ns, const StepParams &p, cudaStream_t st);
+// src [N-1][plane]: the initial phase fields, copied to p.phi (src may be p.phi).
+cudaError_t launch_init(int ns, const StepParams &p, const float *src, cudaStream_t st);
 // A state in motion (velocity.cu): p describes the state set by launch_init
 // (p.phi, p.fout, p.gout, p.mphi); u0 [2][plane] the velocity, u_prev the
 // velocity buffer the first step reads as its previous one, p_scratch one
