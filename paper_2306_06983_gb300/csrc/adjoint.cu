@@ -855,23 +855,35 @@ constexpr int kRevX = 32, kRevY = 8, kRevThreads = kRevX * kRevY;
 inline int rev_blocks(const StepParams &P) { return ((P.nx + kRevX - 1) / kRevX) * ((P.ny + kRevY - 1) / kRevY); }
 
 // Adds the block's sums of K per-thread values to gacc[q][block] in FP64, in
-// a fixed order: thread lane l of a warp sums the values of threads l, l + 32,
-// ..., then the lanes are added pairwise.  (Per-node FP64 sums, read and
+// a fixed order: lane l of a warp sums the values of threads l, l + 32, ...,
+// then the lanes are added, pairwise both.  (Per-node FP64 sums, read and
 // written every step, cost 16 bytes a node and value; FP64 additions are few
 // per SM, so the values meet in shared memory first.)
+// The running sums are read at the start of the kernel (old_sum, the first
+// that the warp adds to), so that nothing waits for them at its end.
 template <int K>
-__device__ __forceinline__ void block_sums(const float (&v)[K], float *s_v, double *gacc, int first)
+__device__ __forceinline__ double old_sum(const double *gacc, int first)
 {
+    const int q = threadIdx.x >> 5;
+    return q < K && (threadIdx.x & 31) == 0 ? gacc[(size_t)(first + q) * gridDim.x + blockIdx.x] : 0.0;
+}
+template <int K>
+__device__ __forceinline__ void block_sums(const float (&v)[K], float *s_v, double *gacc, int first, double old)
+{
+    static_assert(kRevThreads == 256, "eight values a lane");
 #pragma unroll
     for (int q = 0; q < K; ++q) s_v[q * kRevThreads + threadIdx.x] = v[q];
     __syncthreads();
     const int lane = threadIdx.x & 31;
     for (int q = threadIdx.x >> 5; q < K; q += kRevThreads / 32) {
-        double a = (double)s_v[q * kRevThreads + lane];
-#pragma unroll
-        for (int w = 1; w < kRevThreads / 32; ++w) a += (double)s_v[q * kRevThreads + 32 * w + lane];
+        const float *w = s_v + q * kRevThreads + lane;
+        double a = (((double)w[0] + (double)w[32]) + ((double)w[64] + (double)w[96])) +
+                   (((double)w[128] + (double)w[160]) + ((double)w[192] + (double)w[224]));
         for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
-        if (lane == 0) gacc[(size_t)(first + q) * gridDim.x + blockIdx.x] += a;
+        if (lane == 0) {
+            double *sum = gacc + (size_t)(first + q) * gridDim.x + blockIdx.x;
+            *sum = (q < kRevThreads / 32 ? old : *sum) + a;
+        }
     }
 }
 
@@ -883,11 +895,12 @@ __global__ void __launch_bounds__(kRevThreads, NS <= 2 ? 3 : (NS <= 4 ? 2 : 1)) 
     pdl_wait();   // the previous kernel of the sweep has completed
     const int bx = (P.nx + kRevX - 1) / kRevX, by = blockIdx.x / bx;
     const int x = (blockIdx.x - by * bx) * kRevX + threadIdx.x % kRevX, y = by * kRevY + threadIdx.x / kRevX;
+    const double old = old_sum<K>(A.gacc, 0);
     float sums[K];
 #pragma unroll
     for (int q = 0; q < K; ++q) sums[q] = 0.f;
     if (x < P.nx && y < P.ny) rev_collide_node<NS, GATHER, WALLS>(P, T, A, x, y, (unsigned)y * P.nx + x, sums);
-    block_sums<K>(sums, s_v, A.gacc, 0);
+    block_sums<K>(sums, s_v, A.gacc, 0, old);
 }
 
 // rev2 and rev3 on a tile.  rev2 runs on the tile and, for what rev3 gathers,
@@ -918,6 +931,7 @@ __global__ void __launch_bounds__(kRevThreads) rev_source_kernel(const StepParam
             s_l[(3 * p + 2) * RN + r] = __ldg(A.llap + (size_t)p * pl + n);
         }
     };
+    const double old = old_sum<1>(A.gacc, (NS + 1) * NS / 2);
     float pw[NS], sums[1] = {0.f};
     if (own) {
         float d_ph[NS], gx[NS], gy[NS], d_ux, d_uy;
@@ -947,7 +961,7 @@ __global__ void __launch_bounds__(kRevThreads) rev_source_kernel(const StepParam
                                           b, c);
         put((ry + 1) * RX + rx + 1, n, gx, gy);
     }
-    block_sums<1>(sums, s_v, A.gacc, (NS + 1) * NS / 2);   // its barrier also closes s_l
+    block_sums<1>(sums, s_v, A.gacc, (NS + 1) * NS / 2, old);   // its barrier also closes s_l
     if (own) {
         const int c = (ly + 1) * RX + lx + 1;
 #pragma unroll
