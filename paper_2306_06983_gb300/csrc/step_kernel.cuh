@@ -1734,6 +1734,17 @@ cudaError_t launch_step_nst(const StepParams &p, int ty, cudaStream_t st)
     if (e != cudaSuccess) return e;
     if (ty <= 0 && use_patches<NS, MODEL, ST>(p.ny, march_chunks(p, T, slots), vec))
         return launch_patches<NS, MODEL, ST, TAPE>(p, st);
+    // Long marches at N = 5 and 6: many short chunks of narrow strips start
+    // their rows at different times where one wave marches in step (us a step,
+    // one wave / 20 rows of 60 columns: 2048^2 N = 5 340 / 331, N = 6 442 / 415,
+    // 1792^2 267 / 256 and 335 / 319; equal at 44 rows a chunk, slower below,
+    // and slower at N = 7 and 8 on some sizes: 2304^2 N = 8 774 / 803).
+    if constexpr (ST == 0 && !TAPE && (NS == 4 || NS == 5)) {
+        if (ty <= 0 && vec && p.ny > 50 * march_chunks(p, T, slots)) {
+            if ((e = variant_slots<NS, MODEL, 64, ST, true, TAPE>(dev, &slots)) != cudaSuccess) return e;
+            return launch_step_variant<NS, MODEL, 64, ST, true, TAPE>(p, 20, slots, st);
+        }
+    }
     return vec ? launch_step_variant<NS, MODEL, T, ST, true, TAPE>(p, ty, slots, st)
                : launch_step_variant<NS, MODEL, T, ST, false, TAPE>(p, ty, slots, st);
 }
