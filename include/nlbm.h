@@ -203,8 +203,9 @@ int64_t nlbm_kernel_launches(const nlbm_sim *s);
  * down ty rows (>= 1), or ty = 0 (the default) to let the library choose:
  * patches of 16 or 32 columns and 8 rows where marches would be short, else
  * every strip cut into equal row chunks (at least 2 rows) so that the grid
- * is one wave of resident blocks.  Results do not depend on the tile.
- * EINVAL outside those values.  Takes effect on the next nlbm_step(). */
+ * is one wave of resident blocks.  With 16-bit storage the step always runs
+ * on patches.  Results do not depend on the tile.  EINVAL outside those
+ * values.  Takes effect on the next nlbm_step(). */
 nlbm_status nlbm_set_tile(nlbm_sim *s, int32_t tx, int32_t ty);
 nlbm_status nlbm_get_tile(const nlbm_sim *s, int32_t *tx, int32_t *ty);
 
@@ -216,8 +217,9 @@ nlbm_status nlbm_get_tile(const nlbm_sim *s, int32_t *tx, int32_t *ty);
  * nlbm_state_bytes()); keeps the fastest shape.  The result of a step does
  * not depend on the tile (every node is computed by the same code from the
  * same inputs), and the state and step counter are those of the call on
- * return; the trial launches count in nlbm_kernel_launches().  Any output
- * pointer may be NULL.  ENOMEM when the scratch is too small.
+ * return; the trial launches count in nlbm_kernel_launches().  With 16-bit
+ * storage, which has one shape, tx stays and ty = 0 alone is timed.  Any
+ * output pointer may be NULL.  ENOMEM when the scratch is too small.
  * Synchronizes. */
 nlbm_status nlbm_autotune(nlbm_sim *s, void *dev_scratch, size_t scratch_bytes, int32_t steps_per_trial,
                           int32_t *best_tx, int32_t *best_ty, float *best_ms_per_step);

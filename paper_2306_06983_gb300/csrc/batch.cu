@@ -40,14 +40,14 @@ __global__ void __launch_bounds__(T) batch_step_kernel(const StepParams *__restr
         __syncthreads();
         if (s_P.row_window) {
             if (s_P.model == 0)
-                step_tile<NS, 0, T, 0, true>(s_P, tl.x0, tl.y0, tl.ty, smem);
+                step_tile<NS, 0, T, true>(s_P, tl.x0, tl.y0, tl.ty, smem);
             else
-                step_tile<NS, 1, T, 0, true>(s_P, tl.x0, tl.y0, tl.ty, smem);
+                step_tile<NS, 1, T, true>(s_P, tl.x0, tl.y0, tl.ty, smem);
         } else {
             if (s_P.model == 0)
-                step_tile<NS, 0, T, 0, false>(s_P, tl.x0, tl.y0, tl.ty, smem);
+                step_tile<NS, 0, T, false>(s_P, tl.x0, tl.y0, tl.ty, smem);
             else
-                step_tile<NS, 1, T, 0, false>(s_P, tl.x0, tl.y0, tl.ty, smem);
+                step_tile<NS, 1, T, false>(s_P, tl.x0, tl.y0, tl.ty, smem);
         }
         __syncthreads();   // s_k, s_P and the rings are reused by the next tile
     }
@@ -88,7 +88,7 @@ template <int NS, int T>
 cudaError_t configure(int *blocks)
 {
     static_assert(sizeof(StepParams) % sizeof(int) == 0, "parameter block copied as ints");
-    const size_t smem = step_smem_bytes<NS, T, 0, true>();
+    const size_t smem = step_smem_bytes<NS, T, true>();
     // resident blocks per device, 0 until configured (threads that race here
     // compute and store the same value)
     static std::atomic<int> resident[64];
@@ -120,7 +120,7 @@ cudaError_t launch_nt(const StepParams *d_params, const BatchTile *d_tiles, int 
     cudaError_t e = configure<NS, T>(&blocks);
     if (e != cudaSuccess) return e;
     const int grid = ntiles < blocks ? (ntiles > 0 ? ntiles : 1) : blocks;
-    return launch_pdl(batch_step_kernel<NS, T>, dim3(grid), dim3(T), step_smem_bytes<NS, T, 0, true>(), st, d_params,
+    return launch_pdl(batch_step_kernel<NS, T>, dim3(grid), dim3(T), step_smem_bytes<NS, T, true>(), st, d_params,
                       d_tiles, ntiles, d_counters, parity);
 }
 

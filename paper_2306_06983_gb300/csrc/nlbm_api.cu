@@ -555,11 +555,13 @@ nlbm_status nlbm_autotune(nlbm_sim *s, void *dev_scratch, size_t scratch_bytes, 
     static const int kTx[] = {64, 128, 256};
     static const int kTy[] = {0, 8, 12, 16, 20, 24, 32, 48};
     float best = 1e30f;
+    if (s->half()) s->ty = 0;
     int btx = s->tx, bty = s->ty;
     for (int tx : kTx) {
         // a strip of tx - 4 columns; skip widths the lattice cannot fill
-        if (tx > 64 && (tx / 2 - 4) >= s->kp.nx) continue;
+        if (!s->half() && tx > 64 && (tx / 2 - 4) >= s->kp.nx) continue;
         for (int ty : kTy) {
+            if (s->half() && (tx != btx || ty != bty)) continue;   // 16-bit storage has one shape: timed once
             s->tx = tx;
             s->ty = ty;
             for (int k = 0; k <= steps_per_trial && st == NLBM_OK; ++k) {

@@ -207,7 +207,7 @@ __device__ __forceinline__ void sum_pulled(const float *s_F, int WF, int col, fl
     if (NS & 1) sum_pulled_v<float, OWN>(s_F, WF, col, NS - 1, ph, plo, jx, jy);
 }
 
-// Row windows (FP32 storage, nx a multiple of 4, no wall across x).  Each
+// Row windows (nx a multiple of 4, no wall across x).  Each
 // warp stages the rows its 32 ring columns pull from: for every population
 // plane, a window of kWin columns that starts 4 columns left of the warp's
 // first node (so that it is 16-byte aligned) and covers the one-column halo
@@ -489,224 +489,6 @@ __device__ __forceinline__ size_t dev_tail(int NS, int i1, unsigned pl, unsigned
 __device__ __forceinline__ float w_of(int i) { return i == 0 ? 4.f / 9.f : (i < 5 ? 1.f / 9.f : 1.f / 36.f); }
 __device__ __forceinline__ int cx_of(int i) { return (i == 1 || i == 5 || i == 8) ? 1 : (i == 3 || i == 6 || i == 7) ? -1 : 0; }
 __device__ __forceinline__ int cy_of(int i) { return (i == 2 || i == 5 || i == 6) ? 1 : (i == 4 || i == 7 || i == 8) ? -1 : 0; }
-
-// Staging of the 16-bit populations a ring node pulls.  Slots per phase: 0
-// the FP32 rest population, 1..8 the moving deviations, 9 the puller's own
-// phi(t).  A phase pair's word is copied whole into the slots of its even
-// phase.  cp.async moves 4 bytes at least, so for an odd last phase the
-// aligned word holding each 16-bit value is copied and the half is picked in
-// stage A (par bit i: upper half for direction i; nx is even, so every plane
-// starts on a word boundary and the half is the parity of the source node).
-template <int NS>
-__device__ __forceinline__ unsigned prefetch_pull16(const StepParams &P, int x, int y, float *s_F,
-                                                    int WF, int col)
-{
-    unsigned node[9];
-    int dir[9];
-    pull_sources(P, x, y, node, dir);
-    const unsigned pl = P.plane;
-    const unsigned *w32 = (const unsigned *)P.fin;
-    const char *f16 = (const char *)P.fin;
-    unsigned par = 0;
-#pragma unroll
-    for (int i = 1; i < 9; ++i) par |= (node[i] & 1u) << i;
-#pragma unroll
-    for (int p = 0; p < NS; ++p) {
-        cp_async4(s_F + (p * 10) * WF + col, P.f0in + (size_t)p * pl + node[0]);
-        cp_async4(s_F + (p * 10 + 9) * WF + col, P.phi_prev + (size_t)p * pl + node[0]);
-    }
-#pragma unroll
-    for (int q = 0; q < NS / 2; ++q) {
-#pragma unroll
-        for (int i = 1; i < 9; ++i)
-            cp_async4(s_F + (2 * q * 10 + i) * WF + col, (const float *)(w32 + dev_word(q, dir[i] - 1, pl, node[i])));
-    }
-    if (NS & 1) {
-#pragma unroll
-        for (int i = 1; i < 9; ++i) {
-            const size_t e = dev_tail(NS, dir[i] - 1, pl, node[i]);
-            cp_async4(s_F + ((NS - 1) * 10 + i) * WF + col, (const float *)(f16 + ((e * 2) & ~(size_t)3)));
-        }
-    }
-    return par;
-}
-
-// phi and j of one node from its staged 16-bit pull: f_i = w_i phi_own +
-// dev_i (the same FP32 fma the storing node used), summed like sum_pulled.
-template <int NS, int ST, bool OWN>
-__device__ __forceinline__ void sum_pulled16(const float *s_F, int WF, int col, unsigned par,
-                                             float (&ph)[NS], float (&plo)[NS], float (&jx)[NS],
-                                             float (&jy)[NS])
-{
-#pragma unroll
-    for (int p = 0; p + 1 < NS; p += 2) {
-        const float2 own = make_float2(s_F[(p * 10 + 9) * WF + col], s_F[((p + 1) * 10 + 9) * WF + col]);
-        float2 f[9];
-        f[0] = make_float2(s_F[(p * 10) * WF + col], s_F[((p + 1) * 10) * WF + col]);
-#pragma unroll
-        for (int i = 1; i < 9; ++i)
-            f[i] = vfma(vset<float2>(w_of(i)), own, Pack16<ST>::dec2(__float_as_uint(s_F[(p * 10 + i) * WF + col])));
-        float2 a, lo, x, y;
-        pull_moments<float2, OWN>(f, a, lo, x, y);
-        vput(ph, p, a);
-        if (OWN) { vput(plo, p, lo); vput(jx, p, x); vput(jy, p, y); }
-    }
-    if (NS & 1) {
-        constexpr int p = NS - 1;
-        const float own = s_F[(p * 10 + 9) * WF + col];
-        float f[9];
-        f[0] = s_F[(p * 10) * WF + col];
-#pragma unroll
-        for (int i = 1; i < 9; ++i) {
-            const unsigned wd = __float_as_uint(s_F[(p * 10 + i) * WF + col]);
-            const unsigned h = ((par >> i) & 1u) ? (wd >> 16) : (wd & 0xffffu);
-            f[i] = __fmaf_rn(w_of(i), own, Store16<ST>::dec(h));
-        }
-        float a, lo, x, y;
-        pull_moments<float, OWN>(f, a, lo, x, y);
-        ph[p] = a;
-        if (OWN) { plo[p] = lo; jx[p] = x; jy[p] = y; }
-    }
-}
-
-// Row windows of the 16-bit form (nx a multiple of 8, no wall across x).
-// Deviation planes: a window of kWin16 columns starting at the 8-aligned
-// column ws at or left of the warp's first source column, so lane l finds
-// the value pulled along c_i at window column l + o16 - c_ix (o16 = the
-// warp's first node column - ws, 2 or 6): per phase pair and direction 40
-// words (10 pieces of 16 bytes), for an odd last phase 40 16-bit values (5
-// pieces).  FP32 planes read at the node's own column (rest population, own
-// phi) and the source pressure use the kWin windows of the FP32 form.
-// Deviation pieces are copied by lanes 0..29 (group g, piece c), FP32 pieces
-// by lanes 0..26.
-constexpr int kWin16 = 40;
-
-__device__ __forceinline__ void cp_async16_raw(void *dst_smem, const void *src)
-{
-    const unsigned d = (unsigned)__cvta_generic_to_shared(dst_smem);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src) : "memory");
-}
-
-__device__ __forceinline__ unsigned wrap_col(int c, int nx)
-{
-    if (c < 0 || c >= nx) c = ((c % nx) + nx) % nx;
-    return (unsigned)c;
-}
-
-// Copies of what node row y (ring row, image row under a y wall) pulls:
-// the deviation windows s_Dw (phase pairs [NS/2][8][kWin16] words, then an
-// odd last phase [8][kWin16] 16-bit values) and the rest-population and
-// own-phi windows s_Ow [2 NS][kWin] (rest populations first).
-template <int NS>
-__device__ __forceinline__ void stage_pull_rows16(const StepParams &P, int y, int lane, int ws, int xo,
-                                                  unsigned short *s_Dw, float *s_Ow)
-{
-    const unsigned pl = P.plane;
-    if (lane < 30) {
-        const int g = lane / 10, c = lane % 10;
-        int ge;
-        unsigned row;
-        group_source(P, y, g, ge, row);
-        const unsigned *w32 = (const unsigned *)P.fin;
-        unsigned *dw = (unsigned *)s_Dw;
-        const unsigned col4 = row + wrap_col(ws + 4 * c, P.nx);
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            if (g == 0 && k == 0) continue;   // the rest population is FP32
-            const int i1 = group_dir(ge, k) - 1, d1 = group_dir(g, k) - 1;
-#pragma unroll
-            for (int q = 0; q < NS / 2; ++q)
-                cp_async16_raw(dw + (q * 8 + d1) * kWin16 + 4 * c, w32 + dev_word(q, i1, pl, col4));
-            if ((NS & 1) && c < 5) {
-                const unsigned short *f16 = (const unsigned short *)P.fin;
-                cp_async16_raw(s_Dw + (NS / 2) * 16 * kWin16 + d1 * kWin16 + 8 * c,
-                               f16 + dev_tail(NS, i1, pl, row + wrap_col(ws + 8 * c, P.nx)));
-            }
-        }
-    }
-    if (lane < 27) {
-        const int g9 = lane / 9, c9 = lane % 9;
-        const unsigned own = (unsigned)y * (unsigned)P.nx + wrap_col(xo + 4 * c9, P.nx);
-#pragma unroll
-        for (int m = 0; m < (2 * NS + 2) / 3; ++m) {
-            const int q = g9 + 3 * m;
-            if (q < 2 * NS) {
-                const float *src = q < NS ? P.f0in + (size_t)q * pl : P.phi_prev + (size_t)(q - NS) * pl;
-                cp_async16(s_Ow + q * kWin + 4 * c9, src + own);
-            }
-        }
-    }
-}
-
-// Copies of what node row y (an own row) reads for its flow populations:
-// the deviation windows s_Gw [8][kWin16] and the pressure of the rows
-// y - 1, y, y + 1 at the source columns s_Pw [3][kWin] (the own row for a
-// link bounced at a y wall).
-__device__ __forceinline__ void stage_flow_rows16(const StepParams &P, int y, int lane, int ws, int xo,
-                                                  unsigned short *s_Gw, float *s_Pw)
-{
-    if (lane < 15) {
-        const int g = lane / 5, c = lane % 5;
-        int ge;
-        unsigned row;
-        group_source(P, y, g, ge, row);
-        const unsigned short *base = (const unsigned short *)P.gin + (row + wrap_col(ws + 8 * c, P.nx));
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            if (g == 0 && k == 0) continue;   // g_0 is not stored
-            cp_async16_raw(s_Gw + (group_dir(g, k) - 1) * kWin16 + 8 * c,
-                           base + (unsigned)(group_dir(ge, k) - 1) * P.plane);
-        }
-    }
-    if (lane < 27) {
-        const int r9 = lane / 9, c9 = lane % 9;
-        int ys = y - 1 + r9;   // sources with c_iy = +1 sit on row y - 1 (slot 0)
-        if (ys < 0 || ys >= P.ny) ys = P.wall_y ? y : (ys < 0 ? ys + P.ny : ys - P.ny);
-        cp_async16(s_Pw + r9 * kWin + 4 * c9, P.pin + ((unsigned)ys * (unsigned)P.nx + wrap_col(xo + 4 * c9, P.nx)));
-    }
-}
-
-// sum_pulled16 from the warp's windows: f_i = w_i phi_own + dev_i (phases
-// in pairs, see pull_moments).
-template <class V, int NS, int ST, bool OWN>
-__device__ __forceinline__ void sum_pulled16_win_v(const unsigned short *s_Dw, const float *s_Ow, int lane,
-                                                   const WinCols &c, int p, float *ph, float *plo, float *jx,
-                                                   float *jy)
-{
-    const V own = vld<V>(s_Ow + (NS + p) * kWin, kWin, 2 + lane);
-    // the eight deviations: a phase pair's words, or an odd last phase's halves
-    auto dev = [&](int i1, int col) -> V {
-        if constexpr (sizeof(V) == 8) {
-            return Pack16<ST>::dec2(((const unsigned *)s_Dw)[((p / 2) * 8 + i1) * kWin16 + col]);
-        } else {
-            return Store16<ST>::dec(s_Dw[(NS / 2) * 16 * kWin16 + i1 * kWin16 + col]);
-        }
-    };
-    V f[9];
-    f[0] = vld<V>(s_Ow + p * kWin, kWin, 2 + lane);
-    f[1] = vfma(vset<V>(w_of(1)), own, dev(0, c.b - 1));
-    f[2] = vfma(vset<V>(w_of(2)), own, dev(1, c.b));
-    f[3] = vfma(vset<V>(w_of(3)), own, dev(2, c.b + 1));
-    f[4] = vfma(vset<V>(w_of(4)), own, dev(3, c.b));
-    f[5] = vfma(vset<V>(w_of(5)), own, dev(4, c.c5));
-    f[6] = vfma(vset<V>(w_of(6)), own, dev(5, c.c6));
-    f[7] = vfma(vset<V>(w_of(7)), own, dev(6, c.c7));
-    f[8] = vfma(vset<V>(w_of(8)), own, dev(7, c.c8));
-    V a, lo, x, y;
-    pull_moments<V, OWN>(f, a, lo, x, y);
-    vput(ph, p, a);
-    if (OWN) { vput(plo, p, lo); vput(jx, p, x); vput(jy, p, y); }
-}
-template <int NS, int ST, bool OWN>
-__device__ __forceinline__ void sum_pulled16_win(const unsigned short *s_Dw, const float *s_Ow, int lane,
-                                                 const WinCols &c, float (&ph)[NS], float (&plo)[NS],
-                                                 float (&jx)[NS], float (&jy)[NS])
-{
-#pragma unroll
-    for (int p = 0; p + 1 < NS; p += 2)
-        sum_pulled16_win_v<float2, NS, ST, OWN>(s_Dw, s_Ow, lane, c, p, ph, plo, jx, jy);
-    if (NS & 1) sum_pulled16_win_v<float, NS, ST, OWN>(s_Dw, s_Ow, lane, c, NS - 1, ph, plo, jx, jy);
-}
 
 // Eq. (27) on a 3x3 window (rows south, centre, north): the isotropic
 // central gradient and, with LAP, the Laplacian, for one or two phases.
@@ -1281,18 +1063,16 @@ __device__ __forceinline__ float flux_cross(float mx, float my, float ux, float 
 
 // One tile of the fused step: the strip of columns [x0, x0 + T - 4) marching
 // rows [y0, y0 + TY) of the simulation described by P.  smem is the dynamic
-// shared memory of the block (step_smem_bytes gives its size).  VEC: the
-// pulled populations are staged as row windows (nx a multiple of 4, of 8
-// with 16-bit storage, 16-byte aligned planes, no wall across x);
+// shared memory of the block (step_smem_bytes gives its size).  FP32 storage.
+// VEC: the pulled populations are staged as row windows (nx a multiple of 4,
+// 16-byte aligned planes, no wall across x);
 // otherwise every ring thread copies the values its node pulls, 4 bytes at
 // a time.
-template <int NS, int MODEL, int T, int ST, bool VEC = false, bool TAPE = false>
+template <int NS, int MODEL, int T, bool VEC = false, bool TAPE = false>
 __device__ __forceinline__ void step_tile(const StepParams &P, const int x0, const int y0, const int TY,
                                           float *smem)
 {
     constexpr int N = NS + 1;
-    constexpr bool V32 = VEC && ST == 0, V16 = VEC && ST != 0;
-    static_assert(!TAPE || ST == 0, "the adjoint tape is written by the FP32 form");
     // Thread t owns ring column t, lattice column x0 - 2 + t: every thread
     // pulls one phase field in stage A, the inner T - 2 compute m_phi in
     // stage B and the inner T - 4 (the strip) complete their node in stage
@@ -1303,16 +1083,8 @@ __device__ __forceinline__ void step_tile(const StepParams &P, const int x0, con
     float *s_w = s_phi + 5 * NE * T;         // [3][T]       w = m_phi,x u_y - u_x m_phi,y, rows r-1..r+1
     float *s_j = s_w + 3 * T;                // [3][3][NE/2][T][2] j_x, j_y, phi_lo of own nodes
     float *s_F = s_j + 9 * NE * T;           // [9NS][T]     staged pulled f of the next row
-                                             // ([10NS][T] with 16-bit storage, see prefetch_pull16;
-                                             // VEC: [T/32][9NS][kWin] row windows)
+                                             // (VEC: [T/32][9NS][kWin] row windows)
     float *s_G = s_F + (T / 32) * 9 * NS * kWin;   // VEC: [2][T/32][8][kWin] g windows of two rows
-    // VEC with 16-bit storage: [T/32][8NS][kWin16] deviation and [T/32][2NS][kWin]
-    // rest-population / own-phi windows, then per row parity [T/32][8][kWin16] g
-    // deviations and [T/32][3][kWin] pressure rows
-    unsigned short *s_D16 = (unsigned short *)s_F;
-    float *s_O16 = (float *)(s_D16 + (T / 32) * 8 * NS * kWin16);
-    unsigned short *s_G16 = (unsigned short *)(s_O16 + (T / 32) * 2 * NS * kWin);
-    float *s_P16 = (float *)(s_G16 + 2 * (T / 32) * 8 * kWin16);
 
     const int t = threadIdx.x;
     const int We = min(W, P.nx - x0), TYe = min(TY, P.ny - y0);
@@ -1325,24 +1097,18 @@ __device__ __forceinline__ void step_tile(const StepParams &P, const int x0, con
     const int xc = in_ring ? map_axis(x0 - 2 + t, nx, P.wall_x, xflip) : 0;
     const int xg = x0 - 2 + t;                   // lattice x of an own node
 
-    unsigned par_next = 0, par_cur = 0;   // halves of the staged 16-bit words
     // VEC: this lane's window piece and direction group, the (wrapped)
     // lattice column of that piece, and the warp's windows.
     const int lane = t & 31, wc = lane % 9, wg = lane / 9, warp = t >> 5;
-    const bool copier = V32 ? (lane < 27 && 32 * warp < We + 4) : (V16 && 32 * warp < We + 4);
+    const bool copier = VEC && lane < 27 && 32 * warp < We + 4;
     unsigned wcol = 0;
-    if constexpr (V32) {
+    if constexpr (VEC) {
         int c = x0 - 4 + 32 * warp + 4 * wc;
         if (c < 0 || c >= nx) c = ((c % nx) + nx) % nx;   // periodic x: a piece never straddles the edge
         wcol = (unsigned)c;
     }
     float *s_Fw = s_F + warp * 9 * NS * kWin;
     float *s_Gw = s_G + warp * 8 * kWin;   // + (row & 1) * (T / 32) * 8 * kWin
-    // 16-bit windows of this warp: first column of the deviation windows (ws),
-    // of the FP32 windows (xo), and the window column of lane 0's node (o16)
-    const int xo = x0 - 4 + 32 * warp, ws = ((x0 - 3 + 32 * warp) >> 3) * 8, o16 = x0 - 2 + 32 * warp - ws;
-    unsigned short *s_Dw = s_D16 + warp * 8 * NS * kWin16;
-    float *s_Ow = s_O16 + warp * 2 * NS * kWin;
     // The pulled populations of row r+1 are copied into shared memory
     // (cp.async) while rows r..r-2 are computed.  Without VEC each thread
     // only reads the slots it filled itself; with VEC the warp barrier after
@@ -1350,13 +1116,10 @@ __device__ __forceinline__ void step_tile(const StepParams &P, const int x0, con
     {
         bool yflip;
         const int ya = map_axis(y0 - 2, P.ny, P.wall_y, yflip);
-        if constexpr (V32) {
+        if constexpr (VEC) {
             if (copier) stage_pull_rows<NS>(P, ya, wg, wc, wcol, s_Fw);
-        } else if constexpr (V16) {
-            if (copier) stage_pull_rows16<NS>(P, ya, lane, ws, xo, s_Dw, s_Ow);
         } else if (in_ring) {
-            if constexpr (ST == 0) prefetch_pull<NS>(P, xc, ya, s_F, T, t);
-            else par_next = prefetch_pull16<NS>(P, xc, ya, s_F, T, t);
+            prefetch_pull<NS>(P, xc, ya, s_F, T, t);
         }
         cp_async_commit();
     }
@@ -1367,9 +1130,8 @@ __device__ __forceinline__ void step_tile(const StepParams &P, const int x0, con
 #pragma unroll
     for (int p = 0; p < NS; ++p) { Rcx[p] = Rcy[p] = Rnx[p] = Rny[p] = 0.f; }
     float Mcx = 0.f, Mcy = 0.f, Mnx = 0.f, Mny = 0.f;   // m_phi(t)
-    // FP32 storage: phi, grad phi and lap phi of the row stage B evaluated
-    // (Eq. (27)); stage C of the same row reuses them instead of reading the
-    // window again (16-bit storage reads the window there anyway)
+    // phi, grad phi and lap phi of the row stage B evaluated (Eq. (27)); stage
+    // C of the same row reuses them instead of reading the window again
     float PHc[NS], GXc[NS], GYc[NS], LPc[NS], PHn[NS], GXn[NS], GYn[NS], LPn[NS];
 #pragma unroll
     for (int p = 0; p < NS; ++p) PHc[p] = GXc[p] = GYc[p] = LPc[p] = PHn[p] = GXn[p] = GYn[p] = LPn[p] = 0.f;
@@ -1387,8 +1149,6 @@ __device__ __forceinline__ void step_tile(const StepParams &P, const int x0, con
         // (loaded raw; anything computed from them waits until stage C, so
         // that the loads overlap stages A and B)
         float g[9], php[NS], mpx = 0.f, mpy = 0.f;
-        float gps[9];             // 16-bit storage: P of the source node
-        unsigned short gq[9];     // 16-bit storage: stored deviation
         unsigned node = 0;
         const bool do_c = it >= 4 && own;
         if (do_c) {
@@ -1398,15 +1158,8 @@ __device__ __forceinline__ void step_tile(const StepParams &P, const int x0, con
             if constexpr (!VEC) pull_sources(P, xg, y, gnode, gdir);
 #pragma unroll
             for (int i = 1; i < 9; ++i) {
-                if constexpr (VEC) {
-                    // staged as a row window, read in stage C
-                } else if constexpr (ST == 0) {
-                    g[i] = __ldg(P.gin + (unsigned)(gdir[i] - 1) * pl + gnode[i]);
-                } else {
-                    const unsigned short *g16 = (const unsigned short *)P.gin;
-                    gq[i] = __ldg(g16 + (unsigned)(gdir[i] - 1) * pl + gnode[i]);
-                    gps[i] = __ldg(P.pin + gnode[i]);
-                }
+                // VEC: staged as a row window, read in stage C
+                if constexpr (!VEC) g[i] = __ldg(P.gin + (unsigned)(gdir[i] - 1) * pl + gnode[i]);
             }
             node = (unsigned)y * nx + xg;
 #pragma unroll
@@ -1428,7 +1181,6 @@ __device__ __forceinline__ void step_tile(const StepParams &P, const int x0, con
         }
         asm volatile("cp.async.wait_group 0;\n" ::: "memory");   // this row's pulled f landed
         if constexpr (VEC) __syncwarp();
-        par_cur = par_next;
         // ---------------------------------------------------- stage A
         if (in_ring) {
             float ph[NS], plo[NS], jx[NS], jy[NS];
@@ -1436,12 +1188,9 @@ __device__ __forceinline__ void step_tile(const StepParams &P, const int x0, con
                 bool yflip;
                 const int yi = map_axis(ra, P.ny, P.wall_y, yflip);
                 const bool bl = P.wall_y && yi == 0, bh = P.wall_y && yi == P.ny - 1;
-                if constexpr (V32) sum_pulled_win<NS, true>(s_Fw, win_cols(2 + lane, bl, bh), ph, plo, jx, jy);
-                else sum_pulled16_win<NS, ST, true>(s_Dw, s_Ow, lane, win_cols(lane + o16, bl, bh), ph, plo, jx, jy);
-            } else if constexpr (ST == 0) {
-                sum_pulled<NS, true>(s_F, T, t, ph, plo, jx, jy);
+                sum_pulled_win<NS, true>(s_Fw, win_cols(2 + lane, bl, bh), ph, plo, jx, jy);
             } else {
-                sum_pulled16<NS, ST, true>(s_F, T, t, par_cur, ph, plo, jx, jy);
+                sum_pulled<NS, true>(s_F, T, t, ph, plo, jx, jy);
             }
             if (P.wet && (ra < 0 || ra >= P.ny)) wet_ghost<NS>(P, ra, ph);
             float *prow = s_phi + a5 * NE * T;
@@ -1465,8 +1214,7 @@ __device__ __forceinline__ void step_tile(const StepParams &P, const int x0, con
             if (!VEC && it + 1 < TYe + 4) {
                 bool yflip;
                 const int yn = map_axis(ra + 1, P.ny, P.wall_y, yflip);
-                if constexpr (ST == 0) prefetch_pull<NS>(P, xc, yn, s_F, T, t);
-                else par_next = prefetch_pull16<NS>(P, xc, yn, s_F, T, t);
+                prefetch_pull<NS>(P, xc, yn, s_F, T, t);
             }
         }
         if constexpr (VEC) {
@@ -1475,19 +1223,12 @@ __device__ __forceinline__ void step_tile(const StepParams &P, const int x0, con
                 if (it + 1 < TYe + 4) {
                     bool yflip;
                     const int yn = map_axis(ra + 1, P.ny, P.wall_y, yflip);
-                    if constexpr (V32) stage_pull_rows<NS>(P, yn, wg, wc, wcol, s_Fw);
-                    else stage_pull_rows16<NS>(P, yn, lane, ws, xo, s_Dw, s_Ow);
+                    stage_pull_rows<NS>(P, yn, wg, wc, wcol, s_Fw);
                 }
                 // g of the row stage C completes next iteration
                 const int yg = ra - 1;
-                if (it >= 3 && yg < y0 + TYe) {
-                    if constexpr (V32) {
-                        stage_flow_rows(P, yg, wg, wc, wcol, s_Gw + (yg & 1) * (T / 32) * 8 * kWin);
-                    } else {
-                        const int b = (yg & 1) * (T / 32) + warp;
-                        stage_flow_rows16(P, yg, lane, ws, xo, s_G16 + b * 8 * kWin16, s_P16 + b * 3 * kWin);
-                    }
-                }
+                if (it >= 3 && yg < y0 + TYe)
+                    stage_flow_rows(P, yg, wg, wc, wcol, s_Gw + (yg & 1) * (T / 32) * 8 * kWin);
             }
         }
         cp_async_commit();
@@ -1497,14 +1238,10 @@ __device__ __forceinline__ void step_tile(const StepParams &P, const int x0, con
             const int s3 = a3m1;   // row rb = ra - 1
             if (in_flux) {
                 float ph[N], gx[N], gy[N], Rx[NS], Ry[NS], mx, my;
-                if constexpr (ST == 0) {
-                    float lap[N];
-                    window_grad_lap<NS>(s_phi, T, a5m2, a5m1, a5, t, ph, gx, gy, lap);
+                float lap[N];
+                window_grad_lap<NS>(s_phi, T, a5m2, a5m1, a5, t, ph, gx, gy, lap);
 #pragma unroll
-                    for (int p = 0; p < NS; ++p) { PHn[p] = ph[p]; GXn[p] = gx[p]; GYn[p] = gy[p]; LPn[p] = lap[p]; }
-                } else {
-                    window_grad<NS>(s_phi, T, a5m2, a5m1, a5, t, ph, gx, gy);
-                }
+                for (int p = 0; p < NS; ++p) { PHn[p] = ph[p]; GXn[p] = gx[p]; GYn[p] = gy[p]; LPn[p] = lap[p]; }
                 source_terms<NS, MODEL>(P, ph, gx, gy, Rx, Ry);
                 mass_flux<NS>(P, gx, gy, Rx, Ry, mx, my);
                 s_w[s3 * T + t] = ub_s * flux_cross(mx, my, ub_x, ub_y);
@@ -1522,14 +1259,10 @@ __device__ __forceinline__ void step_tile(const StepParams &P, const int x0, con
             const int y = ra - 2;
             const int sm = a5m3, s0 = a5m2, sp = a5m1;
             float ph[N], gx[N], gy[N], lap[N];
-            if constexpr (ST == 0) {
-                close_phases<NS>(PHc, GXc, GYc, LPc, ph, gx, gy, lap);
-            } else {
-                window_grad_lap<NS>(s_phi, T, sm, s0, sp, t, ph, gx, gy, lap);
-            }
+            close_phases<NS>(PHc, GXc, GYc, LPc, ph, gx, gy, lap);
 
             auto load_g = [&](float (&gv)[9]) {
-                if constexpr (V32) {
+                if constexpr (VEC) {
                     const float *gw = s_Gw + (y & 1) * (T / 32) * 8 * kWin;
                     const WinCols wcl = win_cols(2 + lane, P.wall_y && y == 0, P.wall_y && y == P.ny - 1);
                     gv[1] = gw[wcl.b - 1];
@@ -1540,40 +1273,13 @@ __device__ __forceinline__ void step_tile(const StepParams &P, const int x0, con
                     gv[6] = gw[5 * kWin + wcl.c6];
                     gv[7] = gw[6 * kWin + wcl.c7];
                     gv[8] = gw[7 * kWin + wcl.c8];
-                } else if constexpr (ST == 0) {
+                } else {
 #pragma unroll
                     for (int i = 1; i < 9; ++i) gv[i] = g[i];
-                } else {
-                    if constexpr (V16) {
-                        const int b = (y & 1) * (T / 32) + warp;
-                        const unsigned short *gd = s_G16 + b * 8 * kWin16;
-                        const float *pw = s_P16 + b * 3 * kWin;   // rows y - 1, y, y + 1
-                        const bool bl = P.wall_y && y == 0, bh = P.wall_y && y == P.ny - 1;
-                        const WinCols wd = win_cols(lane + o16, bl, bh), wp = win_cols(2 + lane, bl, bh);
-                        gq[1] = gd[wd.b - 1];
-                        gq[2] = gd[kWin16 + wd.b];
-                        gq[3] = gd[2 * kWin16 + wd.b + 1];
-                        gq[4] = gd[3 * kWin16 + wd.b];
-                        gq[5] = gd[4 * kWin16 + wd.c5];
-                        gq[6] = gd[5 * kWin16 + wd.c6];
-                        gq[7] = gd[6 * kWin16 + wd.c7];
-                        gq[8] = gd[7 * kWin16 + wd.c8];
-                        gps[1] = pw[kWin + wp.b - 1];
-                        gps[2] = pw[(bl ? kWin : 0) + wp.b];
-                        gps[3] = pw[kWin + wp.b + 1];
-                        gps[4] = pw[(bh ? kWin : 2 * kWin) + wp.b];
-                        gps[5] = pw[(bl ? kWin : 0) + wp.c5];
-                        gps[6] = pw[(bl ? kWin : 0) + wp.c6];
-                        gps[7] = pw[(bh ? kWin : 2 * kWin) + wp.c7];
-                        gps[8] = pw[(bh ? kWin : 2 * kWin) + wp.c8];
-                    }
-                    // g_i = 3 w_i P(source) + stored deviation
-#pragma unroll
-                    for (int i = 1; i < 9; ++i) gv[i] = __fmaf_rn(3.f * w_of(i), gps[i], Store16<ST>::dec(gq[i]));
                 }
             };
             const OwnRing<NS> own_node{s_j + a3m2 * 3 * NE * T, s_phi, T, t, sm, s0, sp};
-            complete_node<NS, ST, TAPE>(P, node, xg, y, ph, gx, gy, lap, s_w + a3 * T + t, s_w + a3m2 * T + t,
+            complete_node<NS, 0, TAPE>(P, node, xg, y, ph, gx, gy, lap, s_w + a3 * T + t, s_w + a3m2 * T + t,
                                         s_w + a3m1 * T + t, load_g, php, mpx, mpy, Rcx, Rcy, Mcx, Mcy, Ucx, Ucy,
                                         own_node);
         }
@@ -1599,42 +1305,33 @@ __device__ __forceinline__ void step_tile(const StepParams &P, const int x0, con
 }
 
 // Dynamic shared memory of step_tile: phi ring, w ring, own-node j ring and
-// the staging rows (9 slots per phase, 10 with 16-bit storage; VEC: the
-// warps' pull windows and two rows of flow windows).
-template <int NS, int T, int ST, bool VEC = false>
+// the staging rows (9 slots per phase; VEC: the warps' pull windows and two
+// rows of flow windows).
+template <int NS, int T, bool VEC = false>
 constexpr size_t step_smem_bytes()
 {
     constexpr size_t rings = (size_t)T * (14 * ring_even(NS) + 3);   // phi, w and j rings (floats)
-    if (VEC && ST == 0) return sizeof(float) * (rings + (size_t)(T / 32) * kWin * (9 * NS + 16));
-    if (VEC)   // 16-bit deviation windows (2 bytes a value) and FP32 windows
-        return sizeof(float) * rings +
-               (size_t)(T / 32) * (2 * kWin16 * (8 * NS + 16) + sizeof(float) * kWin * (2 * NS + 6));
-    return sizeof(float) * (rings + (size_t)T * (ST == 0 ? 9 : 10) * NS);
+    if (VEC) return sizeof(float) * (rings + (size_t)(T / 32) * kWin * (9 * NS + 16));
+    return sizeof(float) * (rings + (size_t)T * 9 * NS);
 }
 
-// Blocks per SM the step kernel is compiled for.  FP32 storage: three of 128
-// threads (up to 170 registers a thread; measured: the throughput is flat
-// between 12 and 16 resident warps and falls when the registers are squeezed
-// to fit more); from N = 7 on the row windows leave shared memory for two
-// blocks of 128 (or four of 64), so the registers may grow to 255 (2048^2
-// N = 7: 6,602 -> 8,562 MLUPS with 64-thread blocks).  16-bit storage: four
-// of 128 (128 registers), or as many as the shared memory of a block leaves
-// room for (from N = 6 on).
-template <int NS, int T, int ST, bool VEC>
+// Blocks per SM the step kernel is compiled for: three of 128 threads (up to
+// 170 registers a thread; measured: the throughput is flat between 12 and 16
+// resident warps and falls when the registers are squeezed to fit more); from
+// N = 7 on the row windows leave shared memory for two blocks of 128 (or four
+// of 64), so the registers may grow to 255 (2048^2 N = 7: 6,602 -> 8,562
+// MLUPS with 64-thread blocks).
+template <int NS, int T, bool VEC>
 constexpr int step_min_blocks()
 {
-    if (ST == 0) return (NS >= 6 && VEC ? 256 : 384) / T;   // measured best at N = 7, 8 (255 registers)
-    constexpr size_t smem = step_smem_bytes<NS, T, ST, VEC>();
-    constexpr int by_smem = (int)((228u * 1024u) / (smem + 1024u));
-    constexpr int want = 512 / T;
-    return by_smem < 1 ? 1 : (by_smem < want ? by_smem : want);
+    return (NS >= 6 && VEC ? 256 : 384) / T;
 }
 
 // Grid: one block per (strip, row chunk), strips of T - 4 columns, strip
 // index fastest.  TY > 0: chunks of TY rows; TY = 0: chunk k of `chunks`
 // covers rows [k ny / chunks, (k + 1) ny / chunks).
-template <int NS, int MODEL, int T, int ST, bool VEC, bool TAPE = false>
-__global__ void __launch_bounds__(T, (step_min_blocks<NS, T, ST, VEC>()))
+template <int NS, int MODEL, int T, bool VEC, bool TAPE = false>
+__global__ void __launch_bounds__(T, (step_min_blocks<NS, T, VEC>()))
     step_kernel(const StepParams P, const int TY, const int chunks, const int strips)
 {
     extern __shared__ __align__(16) float smem[];
@@ -1649,25 +1346,25 @@ __global__ void __launch_bounds__(T, (step_min_blocks<NS, T, ST, VEC>()))
         ty = (int)((long long)(k + 1) * P.ny / chunks) - y0;
     }
     if (ty <= 0 || y0 >= P.ny) return;
-    step_tile<NS, MODEL, T, ST, VEC, TAPE>(P, s * (T - 4), y0, ty, smem);
+    step_tile<NS, MODEL, T, VEC, TAPE>(P, s * (T - 4), y0, ty, smem);
 }
 
 // Resident blocks of one kernel variant on device dev (the dynamic
 // shared-memory limit, a per-device function attribute, is set on first use).
-template <int NS, int MODEL, int T, int ST, bool VEC, bool TAPE = false>
+template <int NS, int MODEL, int T, bool VEC, bool TAPE = false>
 cudaError_t variant_slots(int dev, int *out)
 {
-    constexpr size_t smem = step_smem_bytes<NS, T, ST, VEC>();
+    constexpr size_t smem = step_smem_bytes<NS, T, VEC>();
     // resident blocks per device, 0 until configured (threads that race here
     // compute and store the same value)
     static std::atomic<int> slots[64];
     int n = slots[dev].load(std::memory_order_acquire);
     if (!n) {
-        cudaError_t e = cudaFuncSetAttribute(step_kernel<NS, MODEL, T, ST, VEC, TAPE>,
+        cudaError_t e = cudaFuncSetAttribute(step_kernel<NS, MODEL, T, VEC, TAPE>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         int per_sm = 0, sms = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, step_kernel<NS, MODEL, T, ST, VEC, TAPE>, T, smem);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, step_kernel<NS, MODEL, T, VEC, TAPE>, T, smem);
         if (e != cudaSuccess) return e;
         e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (e != cudaSuccess) return e;
@@ -1690,16 +1387,16 @@ inline int march_chunks(const StepParams &p, int T, int nslots)
     return chunks < 1 ? 1 : chunks;
 }
 
-template <int NS, int MODEL, int T, int ST, bool VEC, bool TAPE = false>
+template <int NS, int MODEL, int T, bool VEC, bool TAPE = false>
 cudaError_t launch_step_variant(const StepParams &p, int ty, int nslots, cudaStream_t st)
 {
-    constexpr size_t smem = step_smem_bytes<NS, T, ST, VEC>();
+    constexpr size_t smem = step_smem_bytes<NS, T, VEC>();
     const int strips = (p.nx + T - 5) / (T - 4);
     const int chunks = ty > 0 ? (p.ny + ty - 1) / ty : march_chunks(p, T, nslots);
     if (ty < 0) ty = 0;
     const long long blocks = (long long)strips * chunks;
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-    return launch_pdl(step_kernel<NS, MODEL, T, ST, VEC, TAPE>, dim3((unsigned)blocks), dim3(T), smem, st, p, ty,
+    return launch_pdl(step_kernel<NS, MODEL, T, VEC, TAPE>, dim3((unsigned)blocks), dim3(T), smem, st, p, ty,
                       chunks, strips);
 }
 
@@ -1709,54 +1406,58 @@ cudaError_t launch_step_variant(const StepParams &p, int ty, int nslots, cudaStr
 
 namespace nlbm {
 
-// Row windows need nx a multiple of 4 (of 8 with 16-bit storage: rows and
-// planes start on 16-byte boundaries), 16-byte aligned arrays and no wall
-// across x (a wall bounces single columns back, which a window cannot
-// express); they are used whenever they apply, even where their larger
-// shared memory leaves fewer blocks resident (N = 7: two blocks per SM
-// with windows against three with per-node pulls, and the windows are
-// faster).
-template <int NS, int MODEL, int T, int ST, bool TAPE = false>
-cudaError_t launch_step_nst(const StepParams &p, int ty, cudaStream_t st)
+// Row windows need nx a multiple of 4 (rows and planes start on 16-byte
+// boundaries), 16-byte aligned arrays and no wall across x (a wall bounces
+// single columns back, which a window cannot express); they are used whenever
+// they apply, even where their larger shared memory leaves fewer blocks
+// resident (N = 7: two blocks per SM with windows against three with per-node
+// pulls, and the windows are faster).
+template <int NS, int MODEL, int T, bool TAPE = false>
+cudaError_t launch_step_f32(const StepParams &p, int ty, cudaStream_t st)
 {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    uintptr_t a = reinterpret_cast<uintptr_t>(p.fin) | reinterpret_cast<uintptr_t>(p.gin);
-    if (ST != 0)
-        a |= reinterpret_cast<uintptr_t>(p.f0in) | reinterpret_cast<uintptr_t>(p.phi_prev) |
-             reinterpret_cast<uintptr_t>(p.pin);
-    const bool vec = !p.wall_x && p.nx % (ST == 0 ? 4 : 8) == 0 && (a & 15) == 0;
+    const uintptr_t a = reinterpret_cast<uintptr_t>(p.fin) | reinterpret_cast<uintptr_t>(p.gin);
+    const bool vec = !p.wall_x && p.nx % 4 == 0 && (a & 15) == 0;
     int slots = 0;
-    e = vec ? variant_slots<NS, MODEL, T, ST, true, TAPE>(dev, &slots)
-            : variant_slots<NS, MODEL, T, ST, false, TAPE>(dev, &slots);
+    e = vec ? variant_slots<NS, MODEL, T, true, TAPE>(dev, &slots)
+            : variant_slots<NS, MODEL, T, false, TAPE>(dev, &slots);
     if (e != cudaSuccess) return e;
-    if (ty <= 0 && use_patches<NS, MODEL, ST>(p.ny, march_chunks(p, T, slots), vec))
-        return launch_patches<NS, MODEL, ST, TAPE>(p, st);
+    if (ty <= 0 && use_patches<NS, MODEL>(p.ny, march_chunks(p, T, slots), vec))
+        return launch_patches<NS, MODEL, 0, TAPE>(p, st);
     // Long marches at N = 5 and 6: many short chunks of narrow strips start
     // their rows at different times where one wave marches in step (us a step,
     // one wave / 20 rows of 60 columns: 2048^2 N = 5 340 / 331, N = 6 442 / 415,
     // 1792^2 267 / 256 and 335 / 319; equal at 44 rows a chunk, slower below,
     // and slower at N = 7 and 8 on some sizes: 2304^2 N = 8 774 / 803).
-    if constexpr (ST == 0 && !TAPE && (NS == 4 || NS == 5)) {
+    if constexpr (!TAPE && (NS == 4 || NS == 5)) {
         if (ty <= 0 && vec && p.ny > 50 * march_chunks(p, T, slots)) {
-            if ((e = variant_slots<NS, MODEL, 64, ST, true, TAPE>(dev, &slots)) != cudaSuccess) return e;
-            return launch_step_variant<NS, MODEL, 64, ST, true, TAPE>(p, 20, slots, st);
+            if ((e = variant_slots<NS, MODEL, 64, true, TAPE>(dev, &slots)) != cudaSuccess) return e;
+            return launch_step_variant<NS, MODEL, 64, true, TAPE>(p, 20, slots, st);
         }
     }
-    return vec ? launch_step_variant<NS, MODEL, T, ST, true, TAPE>(p, ty, slots, st)
-               : launch_step_variant<NS, MODEL, T, ST, false, TAPE>(p, ty, slots, st);
+    return vec ? launch_step_variant<NS, MODEL, T, true, TAPE>(p, ty, slots, st)
+               : launch_step_variant<NS, MODEL, T, false, TAPE>(p, ty, slots, st);
 }
 
 template <int NS, int MODEL, int ST>
 cudaError_t launch_step_ns(const StepParams &p, int tx, int ty, cudaStream_t st)
 {
-    switch (tx) {
-    case 64: return launch_step_nst<NS, MODEL, 64, ST>(p, ty, st);
-    case 128: return launch_step_nst<NS, MODEL, 128, ST>(p, ty, st);
-    case 256: return launch_step_nst<NS, MODEL, 256, ST>(p, ty, st);
-    default: return cudaErrorInvalidValue;
+    if constexpr (ST != 0) {
+        // 16-bit storage runs on patches at every size: its marches, bound by
+        // instruction issue, were slower (us a step, march / patches, Model
+        // B: 256^2 N = 5 17.0 / 8.5, 2048^2 N = 3 222 / 185, N = 5 342 / 331, N
+        // = 8 779 / 644; with the best explicit tile 215, 335 and 780)
+        return launch_patches<NS, MODEL, ST, false>(p, st);
+    } else {
+        switch (tx) {
+        case 64: return launch_step_f32<NS, MODEL, 64>(p, ty, st);
+        case 128: return launch_step_f32<NS, MODEL, 128>(p, ty, st);
+        case 256: return launch_step_f32<NS, MODEL, 256>(p, ty, st);
+        default: return cudaErrorInvalidValue;
+        }
     }
 }
 

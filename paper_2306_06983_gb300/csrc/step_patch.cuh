@@ -288,24 +288,21 @@ cudaError_t launch_patches(const StepParams &p, cudaStream_t st)
     return launch_patch_variant<NS, MODEL, ST, 16, 8, kNarrowMin, TAPE>(p, st);
 }
 
-// Whether a step runs on patches rather than as a march of `chunks` row
+// Whether an FP32 step runs on patches rather than as a march of `chunks` row
 // chunks; windows: the march would stage row windows.  A march costs 6 extra
 // rows a chunk, a patch 0.7 to 0.9 extra pulls and a third of the sources per
-// node (FP32, us a step, march / patches, rows a chunk; Model B: 64^2 N = 3
-// 6.4 / 3.5, 2 rows; 256^2 N = 5 15.7 / 8.0, 2; 512^2 N = 5 32.0 / 24.8, 6, N =
-// 8 56.4 / 52.0, 8; 1024^2 N = 5 94.2 / 91.5, 20, N = 7 141.6 / 140.8, 31;
-// 2048^2 N = 5 340 / 366, 78, N = 8 651 / 683).  Ahead at every size: N = 3
-// (2048^2 200 / 192), Model A at N = 5 (339 / 330) and N = 8 (634 / 599, 1024^2
-// 172 / 158); 16-bit storage, whose marches are bound by instruction issue
-// (2048^2 N = 5 342 / 331, N = 3 222 / 185, N = 8 779 / 630); and, where
-// patches are wide, lattices that march without row windows (1021^2 N = 8 210
-// / 185, 2045^2 N = 3 221 / 209, N = 8 761 / 700; narrow patches lose there at
-// size, N = 5 380 / 454).
-template <int NS, int MODEL, int ST>
+// node (us a step, march / patches, rows a chunk; Model B: 64^2 N = 3 6.4 /
+// 3.5, 2 rows; 256^2 N = 5 15.7 / 8.0, 2; 512^2 N = 5 32.0 / 24.8, 6, N = 8 56.4
+// / 52.0, 8; 1024^2 N = 5 94.2 / 91.5, 20, N = 7 141.6 / 140.8, 31; 2048^2 N = 5
+// 340 / 366, 78, N = 8 651 / 683).  Ahead at every size: N = 3 (2048^2 200 /
+// 192), Model A at N = 5 (339 / 330) and N = 8 (634 / 599, 1024^2 172 / 158);
+// and, where patches are wide, lattices that march without row windows (1021^2
+// N = 8 210 / 185, 2045^2 N = 3 221 / 209, N = 8 761 / 700; narrow patches lose
+// there at size, N = 5 380 / 454).
+template <int NS, int MODEL>
 inline bool use_patches(int ny, int chunks, bool windows)
 {
-    if (ST != 0 || NS == 2 || (MODEL == 0 && (NS == 4 || NS == 7)) || (!windows && NS > 1 && wide_patches<NS, MODEL, ST>()))
-        return true;
+    if (NS == 2 || (MODEL == 0 && (NS == 4 || NS == 7)) || (!windows && NS > 1 && wide_patches<NS, MODEL, 0>())) return true;
     return ny <= 24 * chunks;
 }
 

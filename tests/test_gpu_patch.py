@@ -48,17 +48,12 @@ def test_patches_equal_marches(nx, ny, wall_x, wall_y, N, model, n):
     p, phi0 = W.random_smooth(nx, ny, N, seed=nx + ny, model=model, model_a_n=n, wall_x=bool(wall_x),
                               wall_y=bool(wall_y), n_disks=4)
     p = dict(p, gx=1e-6, gy=-2e-6)
-    for storage in ("f32", "bf16", "f16"):
-        if storage != "f32" and nx % 2:
-            continue
-        q = dict(p, storage=storage)
-        assert state(q, phi0, None) == state(q, phi0, (64, 5)), (storage,)
+    assert state(p, phi0, None) == state(p, phi0, (64, 5))
 
 
-@pytest.mark.parametrize("storage", ["f32", "bf16"])
-def test_patches_equal_marches_wetting_walls(storage):
+def test_patches_equal_marches_wetting_walls():
     p, phi0 = W.compound_droplet(60.0, nx=100, ny=50, R=20.0)
-    p = dict(p, storage=storage, wall_cos=[0.3, 0.5, -0.2, 0.1])
+    p = dict(p, wall_cos=[0.3, 0.5, -0.2, 0.1])
     assert state(p, phi0, None) == state(p, phi0, (128, 7))
 
 
