@@ -298,12 +298,13 @@ cudaError_t launch_patches(const StepParams &p, cudaStream_t st)
 // 192), Model A at N = 5 (339 / 330) and N = 8 (634 / 599, 1024^2 172 / 158);
 // and, where patches are wide, lattices that march without row windows (1021^2
 // N = 8 210 / 185, 2045^2 N = 3 221 / 209, N = 8 761 / 700; narrow patches lose
-// there at size, N = 5 380 / 454).
+// there at size, N = 5 380 / 454).  N = 2, with the least work to repeat a
+// row, turns at fewer rows (1021^2, 10 rows: 43 / 46; 512^2, 3: 16.4 / 10.4).
 template <int NS, int MODEL>
 inline bool use_patches(int ny, int chunks, bool windows)
 {
     if (NS == 2 || (MODEL == 0 && (NS == 4 || NS == 7)) || (!windows && NS > 1 && wide_patches<NS, MODEL, 0>())) return true;
-    return ny <= 24 * chunks;
+    return ny <= (NS == 1 ? 8 : 24) * chunks;
 }
 
 }  // namespace nlbm
