@@ -61,33 +61,31 @@ def bytes_per_lup(N: int, storage: str = "f32") -> int:
     return 2 * (2 * (8 * (N - 1) + 8) + 4 * (N - 1) + 4 * ((N - 1) + 5))
 
 
-def adjoint_bytes_per_lup(N: int) -> dict:
+def adjoint_bytes_per_lup(N: int, kept: float = 0.0) -> dict:
     """Algorithmic HBM bytes of one differentiated lattice update (Model B,
-    FP32; NS = N - 1 solved phases, NP = N(N-1)/2 tension pairs), each field
-    a pass reads or writes counted once per pass:
-    forward step 8(10N + 2); reverse step = the taping rebuild (a forward
-    step that also writes 8 NS + 13 tape floats) and four passes:
-    1 collision: 8 NS + 12 tape, NS + 4 state and 10 NS + 12 seed floats
-      read, 9 NS + 16 adjoint floats written, NP + 1 FP64 sums updated;
-    2 source: 10 NS + 10 floats read, 3 NS + 2 written, one FP64 sum updated;
-    3 stencil: 4 NS read, NS written;
-    4 pull: 3 NS + 8 read, 9 NS + 8 written."""
-    NS, NP = N - 1, N * (N - 1) // 2
-    fwd = 8 * (10 * N + 2)
-    tape = fwd + 4 * (8 * NS + 13)
-    collide = 4 * ((8 * NS + 12) + (NS + 4) + (10 * NS + 12) + (9 * NS + 16)) + 16 * (NP + 1)
-    source = 4 * ((10 * NS + 10) + (3 * NS + 2)) + 16
-    stencil = 4 * (4 * NS + NS)
-    pull = 4 * ((3 * NS + 8) + (9 * NS + 8))
-    return {"forward": fwd, "reverse": tape + collide + source + stencil + pull,
-            "reverse_parts": {"taping_rebuild": tape, "collision": collide, "source": source,
-                              "stencil": stencil, "pull": pull}}
+    FP32; NS = N - 1 solved phases), each field a pass reads or writes counted
+    once per pass; kept: the share of the steps that are taped by the forward
+    (its last segment) instead of being rebuilt in the sweep.
+    Forward step 8(10N + 2), and 8 NS + 13 tape floats where it tapes; reverse
+    step = the taping rebuild (a forward step that also writes the tape) and
+    two passes:
+    1 collision: 8 NS + 12 tape, NS + 4 state, NS + 4 seed and 3 NS + 8
+      gathered floats read, 9 NS + 16 written;
+    2 source and stencils: 9 NS + 10 floats read, NS + 2 written."""
+    NS = N - 1
+    step, tape = 8 * (10 * N + 2), 4 * (8 * NS + 13)
+    fwd = step + kept * tape
+    rebuild = (1.0 - kept) * (step + tape)
+    collide = 4 * ((8 * NS + 12) + (NS + 4) + (NS + 4) + (3 * NS + 8) + (9 * NS + 16))
+    source = 4 * ((9 * NS + 10) + (NS + 2))
+    return {"forward": round(fwd, 1), "reverse": round(rebuild + collide + source, 1),
+            "reverse_parts": {"taping_rebuild": round(rebuild, 1), "collision": collide, "source": source}}
 
 
 def kernel_sources_digest() -> str:
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_2306_06983_gb300", "csrc")
-    for name in ("step_kernel.cuh", "nlbm_internal.cuh"):
+    for name in ("step_kernel.cuh", "step_patch.cuh", "nlbm_internal.cuh"):
         with open(os.path.join(csrc, name), "rb") as f:
             h.update(f.read())
     return h.hexdigest()[:16]
@@ -514,7 +512,7 @@ def measure_adjoint(timed, n=256, peak=None, model="B"):
     run.close()
     fwd, bwd = float(np.median(fwds)), float(np.median(bwds))
     nodes = n * n
-    ab = adjoint_bytes_per_lup(N)
+    ab = adjoint_bytes_per_lup(N, kept=every / T)
     roof = None
     if peak:
         gbs = (ab["forward"] + ab["reverse"]) * nodes * T / ((fwd + bwd) / 1e3) / 1e9
