@@ -10,6 +10,8 @@
 #include <new>
 #include <vector>
 
+#include <cuda.h>
+
 #include "../../include/nlbm.h"
 #include "nlbm_internal.cuh"
 #include "adjoint.cuh"
@@ -75,6 +77,41 @@ void set_err(char *buf, const char *fmt, ...)
 }
 
 bool finite_pos(double v) { return std::isfinite(v) && v > 0.0; }
+
+// Whether a kernel may read the caller's [src, src + bytes) where it lies: a
+// float array within one allocation of the current device's own memory.
+// Everything else that a copy takes (memory of another device, managed or
+// host memory, an odd address) or refuses (a range beyond its allocation) is
+// left to the copy.
+bool device_readable(const void *src, size_t bytes)
+{
+    using Get = CUresult (*)(unsigned, CUpointer_attribute *, void **, CUdeviceptr);
+    static const Get get = [] {
+        void *f = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        const cudaError_t e = cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 12000, cudaEnableDefault, &q);
+        if (e != cudaSuccess) cudaGetLastError();
+        return e == cudaSuccess && q == cudaDriverEntryPointSuccess ? reinterpret_cast<Get>(f) : nullptr;
+    }();
+    if (!get || ((uintptr_t)src & (sizeof(float) - 1))) return false;
+    unsigned type = 0, managed = 0;   // left 0 for an address the driver does not know
+    int ordinal = -1, device = -1;
+    CUdeviceptr start = 0;
+    size_t size = 0;
+    CUpointer_attribute what[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED,
+                                  CU_POINTER_ATTRIBUTE_DEVICE_ORDINAL, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                                  CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    void *out[] = {&type, &managed, &ordinal, &start, &size};
+    if (get(5, what, out, (CUdeviceptr)src) != CUDA_SUCCESS || type != CU_MEMORYTYPE_DEVICE || managed) return false;
+    if (cudaGetDevice(&device) != cudaSuccess || ordinal != device) return false;
+    const CUdeviceptr at = (CUdeviceptr)src;
+    return at >= start && at - start <= size && bytes <= size - (at - start);
+}
+
+bool overlap(const void *a, size_t na, const void *b, size_t nb)
+{
+    return (uintptr_t)a < (uintptr_t)b + nb && (uintptr_t)b < (uintptr_t)a + na;
+}
 
 // Validates the problem statement; fills the derived kernel parameters.
 nlbm_status validate(const nlbm_params *p, StepParams *kp, char *err)
@@ -245,6 +282,20 @@ StepParams step_params(const nlbm_sim *s, int a, int b)
     return kp;
 }
 
+// Where the initial state's kernel reads the caller's phase fields from:
+// dev_phi itself, or, where it may not be read in place or lies in memory
+// ([own, own + own_bytes)) that the kernel writes, the state's phi planes,
+// copied there first.
+cudaError_t initial_fields(const float *dev_phi, float *phi, size_t bytes, const void *own, size_t own_bytes,
+                           cudaStream_t stream, const float **src)
+{
+    *src = dev_phi;
+    if (dev_phi == phi || (!overlap(dev_phi, bytes, own, own_bytes) && device_readable(dev_phi, bytes)))
+        return cudaSuccess;
+    *src = phi;
+    return cudaMemcpyAsync(phi, dev_phi, bytes, cudaMemcpyDeviceToDevice, stream);
+}
+
 // Initial state into the buffers of state c from the phase fields src.
 cudaError_t launch_initial_state(nlbm_sim *s, int c, const float *src)
 {
@@ -320,7 +371,11 @@ nlbm_status nlbm_create(const nlbm_params *p, void *dev_workspace, size_t worksp
 nlbm_status nlbm_set_phi(nlbm_sim *s, const float *dev_phi)
 {
     if (!s || !dev_phi) return NLBM_EINVAL;
-    cudaError_t e = launch_initial_state(s, s->cur, dev_phi);
+    const float *src;
+    cudaError_t e = initial_fields(dev_phi, s->phi(s->cur), sizeof(float) * s->ns * s->plane, s->ws, s->L.total,
+                                   s->stream, &src);
+    if (e != cudaSuccess) return cuda_fail(s, e, "copy of the initial phase fields");
+    e = launch_initial_state(s, s->cur, src);
     if (e != cudaSuccess) return cuda_fail(s, e, "init kernel");
     s->launches++;
     s->steps = 0;
@@ -1077,6 +1132,7 @@ struct nlbm_adjoint {
     size_t plane, state_floats;
     cudaStream_t stream;
     char *ws;
+    size_t ws_bytes;
     float *ckpt;               // [nckpt][state]
     float *seg;                // [every + 1][state]
     float *tapes;              // [every][tape] the rebuilt segment's tapes
@@ -1354,6 +1410,7 @@ nlbm_status nlbm_adjoint_create(const nlbm_params *p, int32_t nsteps, int32_t ch
     a->state_floats = adj_state_floats(a->ns, a->plane);
     a->stream = (cudaStream_t)cuda_stream;
     a->ws = ws;
+    a->ws_bytes = L.total;
     a->ckpt = (float *)(ws + L.ckpt);
     a->seg = (float *)(ws + L.seg);
     a->tapes = (float *)(ws + L.tapes);
@@ -1417,7 +1474,10 @@ nlbm_status nlbm_adjoint_forward(nlbm_adjoint *a, const float *dev_phi0, float *
     kp.uin = kp.uout;             // one velocity buffer in a record
     kp.phi = kp.uout + pl * 2;
     kp.pout = s->P(0);
-    cudaError_t e = launch_init(ns, kp, dev_phi0, a->stream);
+    const float *src;
+    cudaError_t e = initial_fields(dev_phi0, kp.phi, sizeof(float) * pl * ns, a->ws, a->ws_bytes, a->stream, &src);
+    if (e != cudaSuccess) return adj_fail(a, e, "copy of the initial phase fields");
+    e = launch_init(ns, kp, src, a->stream);
     if (e != cudaSuccess) return adj_fail(a, e, "initial state");
     s->launches++;
     a->forward_done = false;
