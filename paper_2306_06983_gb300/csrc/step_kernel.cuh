@@ -604,9 +604,11 @@ __device__ __forceinline__ float inv_norm2(float n2, float delta2)
 }
 
 // Model A weight max(phi, 0)^n, integer n by multiplication from the left.  n
-// = 3 and 4 without the loop (1500^2 N = 3, n = 3: 116.7 -> 113.2 us a step),
-// but for N >= 7, where the longer chain costs registers that are not there
-// (1024^2 N = 8, n = 1: 158 -> 165).
+// = 1 and 2 leave before the longer chain, which has no loop (us a step, loop /
+// one chain of predicated products / this: 2048^2 N = 6 n = 1 427 / 420 / 408, n
+// = 3 465 / 420 / 414, n = 6 480 / 434 / 414; 1500^2 N = 6 n = 1 235 / 239 / 232, N =
+// 3 n = 1 113.0 / 114.0 / 113.2), but for N >= 7, where the longer chain costs
+// registers that are not there (1024^2 N = 8, n = 1: 158 -> 165).
 template <int NS>
 __device__ __forceinline__ float model_a_weight(const StepParams &P, float ph)
 {
@@ -619,12 +621,16 @@ __device__ __forceinline__ float model_a_weight(const StepParams &P, float ph)
             for (int k = 1; k < P.model_n_int; ++k) wq *= pc;
             return wq;
         }
-    } else if (P.model_n_int > 0) {
-        float wq = pc;
-        if (P.model_n_int > 1) wq *= pc;
-        if (P.model_n_int > 2) wq *= pc;
-        if (P.model_n_int > 3) wq *= pc;
-        for (int k = 4; k < P.model_n_int; ++k) wq *= pc;
+    } else if (P.model_n_int > 0) {   // at most 8
+        float wq = P.model_n_int > 1 ? pc * pc : pc;
+        if (P.model_n_int > 2) {
+            wq *= pc;
+            if (P.model_n_int > 3) wq *= pc;
+            if (P.model_n_int > 4) wq *= pc;
+            if (P.model_n_int > 5) wq *= pc;
+            if (P.model_n_int > 6) wq *= pc;
+            if (P.model_n_int > 7) wq *= pc;
+        }
         return wq;
     }
     return powf(pc, P.model_n);
