@@ -303,7 +303,8 @@ nlbm_status nlbm_batch_phase_mass(nlbm_batch *b, int32_t sim, double *host_mass)
 /* Tile shape of the ensemble kernel: tx threads per block (64, 128, 256) and
  * ty rows per tile (>= 1): strips of tx - 4 columns marched down ty rows, or,
  * with 128 or 256 threads and ty = 8, patches of tx / 8 columns computed at
- * once; ty = 0 (the default) lets the library choose (patches of 32 columns).
+ * once; ty = 0 (the default) lets the library choose: patches of 32 columns,
+ * or, for members large enough, marches of 32 rows.
  * Results do not depend on the shape.  Rebuilds the tile table
  * (synchronizes).  get_tile also returns the tile count. */
 nlbm_status nlbm_batch_set_tile(nlbm_batch *b, int32_t tx, int32_t ty);

@@ -1,4 +1,4 @@
-// Ensemble of independent simulations in one persistent launch per step.
+// Ensemble of independent simulations in one launch per step.
 //
 // Every simulation keeps its own state and parameter block (StepParams, in
 // device memory); the host builds a table of tiles over all of them, largest
@@ -136,7 +136,33 @@ cudaError_t launch_n(int tx, const StepParams *d_params, const BatchTile *d_tile
     }
 }
 
+template <int NS>
+cudaError_t march_blocks(int tx, int *blocks)
+{
+    switch (tx) {
+    case 64: return configure<NS, 64>(blocks);
+    case 128: return configure<NS, 128>(blocks);
+    case 256: return configure<NS, 256>(blocks);
+    default: return cudaErrorInvalidValue;
+    }
+}
+
 }  // namespace
+
+cudaError_t batch_march_blocks(int ns, int tx, int *blocks, int *sms)
+{
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    switch (ns) {
+#define NLBM_CASE(K) \
+    case K: return march_blocks<K>(tx, blocks);
+        NLBM_CASE(1) NLBM_CASE(2) NLBM_CASE(3) NLBM_CASE(4) NLBM_CASE(5) NLBM_CASE(6) NLBM_CASE(7)
+#undef NLBM_CASE
+    default: return cudaErrorInvalidValue;
+    }
+}
 
 template <int NS>
 cudaError_t launch_batch_patches_n(int px, const StepParams *d_params, const BatchTile *d_tiles, int ntiles,

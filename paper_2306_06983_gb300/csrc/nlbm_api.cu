@@ -674,6 +674,7 @@ struct nlbm_batch {
     int *d_counters;                     // [2]
     int cur;                             // state parity shared by every simulation
     int tx, ty;
+    int px, rows;                        // the tiles they give, see choose_tiles()
     cudaGraphExec_t graph;               // two steps (parity 0 then 1), no P output
     bool graph_ok;
     int64_t steps, launches;
@@ -699,20 +700,6 @@ size_t worst_tiles(const nlbm_params *p, int count)
         t += std::max((size_t)((p[k].nx + 59) / 60) * (size_t)p[k].ny,
                       (size_t)((p[k].nx + 15) / 16) * (size_t)((p[k].ny + 7) / 8));
     return t;
-}
-
-// Columns of the ensemble's patches (of 8 rows), 0 where it marches rows:
-// with the library's own choice (ty = 0) wide patches, and tiles of 8 rows
-// are patches of tx threads.  Members are small, so a march repeats its 6
-// pre-roll rows often and its last strip is narrow (us a step, march 128 x 32
-// / best march / narrow / wide patches: 64 lenses of 512 x 256 to 128 x 64,
-// N = 3, 228 / 215 / 233 / 195; 8 of them 78 / 44 / 38 / 33; 32 members N = 5
-// 304 / 292 / 260 / 250; 16 members N = 8 413 / 331 / 253 / 242; four of
-// 1024^2, N = 5 406 / 397 / 406 / 399).
-int batch_patch_columns(int tx, int ty)
-{
-    if (ty == 0) return 32;
-    return ty == 8 && tx > 64 ? tx / 8 : 0;
 }
 
 nlbm_status batch_layout(const nlbm_params *p, int count, BatchLayout *B, char *err)
@@ -762,11 +749,70 @@ nlbm_status batch_fail(nlbm_batch *b, cudaError_t e, const char *what)
     return NLBM_ECUDA;
 }
 
+// Whether the pulls of a member's march are staged as row windows: the same
+// condition as the single-simulation launcher's.
+bool row_windows(const StepParams &kp)
+{
+    return !kp.wall_x && kp.nx % 4 == 0 &&
+           ((reinterpret_cast<uintptr_t>(kp.fin) | reinterpret_cast<uintptr_t>(kp.gin)) & 15) == 0;
+}
+
+// Tiles for the current tx and ty: px > 0 patches of px columns and 8 rows,
+// px = 0 strips of tx - 4 columns marched down `rows` rows.
+//
+// ty = 8 with more than 64 threads: patches of those threads; other ty > 0: a
+// march.  ty = 0: the library's choice, wide patches unless a march of 32
+// rows costs less.  Patches win on small members, whose marches repeat their
+// 6 pre-roll rows often and end in narrow strips (us a step, march 128 x 32 /
+// best march / narrow / wide patches: 64 lenses of 512 x 256 to 128 x 64, N =
+// 3, 228 / 215 / 233 / 195; 8 of them 78 / 44 / 38 / 33; 32 members N = 5 304 /
+// 292 / 260 / 250; 16 members N = 8 413 / 331 / 253 / 242).  On large ones a
+// march spends `gain` of a patch's time on a node of its tiles (strips padded
+// to tx - 4 columns, 6 rows more a tile), and part of its last wave idles
+// (N = 5, march / wide patches: 2 of 2048^2 713 / 790, 3 of 1536^2 625 / 673, 2
+// of 1280^2 293 / 321, but 1 of 1536^2 274 / 232; N = 3: 4 of 2048^2 785 / 832,
+// 1 of 2048^2 221 / 216).  Without row windows it gains less, and at N = 8
+// nothing.  Over 160 ensembles of 0.4 to 17 million nodes at N = 2..8 the worse
+// form is taken by at most 2.5 %, 5 % for 3 of 1536^2 at N = 2.
+cudaError_t choose_tiles(nlbm_batch *b)
+{
+    b->px = b->ty == 8 && b->tx > 64 ? b->tx / 8 : 0;
+    b->rows = b->ty;
+    if (b->ty > 0) return cudaSuccess;
+    static const double kGain[2][kMaxPhases - 1] = {{.91, 1., 1., .91, .91, .91, 1.}, {.88, .90, .89, .83, .90, .92, 1.}};
+    const int W = b->tx - 4;
+    double nodes = 0., march = 0., gain = 0.;
+    long long tiles = 0;
+    for (const nlbm_sim *s : b->sims) {
+        const int strips = (s->kp.nx + W - 1) / W, chunks = (s->kp.ny + 31) / 32;
+        const double g = kGain[row_windows(step_params(s, 0, 1))][b->ns - 1];
+        nodes += (double)s->plane;
+        march += g * strips * W * (s->kp.ny + 6. * chunks) * (32. / 38.);
+        gain = std::max(gain, g);
+        tiles += (long long)strips * chunks;
+    }
+    b->px = 32;
+    b->rows = 8;
+    if (march >= nodes) return cudaSuccess;
+    int resident = 0, sms = 0;
+    const cudaError_t e = batch_march_blocks(b->ns, b->tx, &resident, &sms);
+    if (e != cudaSuccess) return e;
+    const double idle = (double)((resident - tiles % resident) % resident);
+    march += gain * std::min(0.68 * sms, sms / 6. + 0.5 * idle) * W * 32.;
+    if (march < nodes) {
+        b->px = 0;
+        b->rows = 32;
+    }
+    return cudaSuccess;
+}
+
 // Tile table for the current tile shape: every strip and row chunk of every
 // simulation, the largest simulations first (so the last tiles are small).
 nlbm_status build_tiles(nlbm_batch *b)
 {
-    const int px = batch_patch_columns(b->tx, b->ty), W = px ? px : b->tx - 4;
+    cudaError_t e = choose_tiles(b);
+    if (e != cudaSuccess) return batch_fail(b, e, "choice of the tiles");
+    const int W = b->px ? b->px : b->tx - 4;
     std::vector<int> order(b->count);
     for (int k = 0; k < b->count; ++k) order[k] = k;
     std::stable_sort(order.begin(), order.end(), [&](int a, int c) {
@@ -776,7 +822,7 @@ nlbm_status build_tiles(nlbm_batch *b)
     for (int k : order) {
         const nlbm_sim *s = b->sims[k];
         const int nx = s->kp.nx, ny = s->kp.ny;
-        int ty = px ? 8 : b->ty;
+        int ty = b->rows;
         if (ty > ny) ty = ny;
         for (int y0 = 0; y0 < ny; y0 += ty)
             for (int x0 = 0; x0 < nx; x0 += W) t.push_back(BatchTile{k, x0, y0, ty});
@@ -785,7 +831,7 @@ nlbm_status build_tiles(nlbm_batch *b)
         set_err(b->err, "tile table of %zu entries exceeds the %zu reserved", t.size(), b->max_tiles);
         return NLBM_EINVAL;
     }
-    cudaError_t e = cudaMemcpyAsync(b->d_tiles, t.data(), sizeof(BatchTile) * t.size(), cudaMemcpyHostToDevice,
+    e = cudaMemcpyAsync(b->d_tiles, t.data(), sizeof(BatchTile) * t.size(), cudaMemcpyHostToDevice,
                                     b->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);   // t is a host temporary
     if (e != cudaSuccess) return batch_fail(b, e, "upload of the tile table");
@@ -800,9 +846,7 @@ nlbm_status upload_params(nlbm_batch *b)
     for (int par = 0; par < 2; ++par)
         for (int k = 0; k < b->count; ++k) {
             StepParams kp = step_params(b->sims[k], par, par ^ 1);
-            // the same condition as the single-simulation launcher's
-            kp.row_window = !kp.wall_x && kp.nx % 4 == 0 &&
-                            ((reinterpret_cast<uintptr_t>(kp.fin) | reinterpret_cast<uintptr_t>(kp.gin)) & 15) == 0;
+            kp.row_window = row_windows(kp);
             kp.pout = nullptr;
             h[(size_t)(2 * par) * b->count + k] = kp;
             kp.pout = b->sims[k]->P(0);
@@ -820,8 +864,7 @@ nlbm_status upload_params(nlbm_batch *b)
 cudaError_t batch_launch(nlbm_batch *b, int parity, bool with_p)
 {
     const StepParams *tab = b->d_params + (size_t)(2 * parity + (with_p ? 1 : 0)) * b->count;
-    const int px = batch_patch_columns(b->tx, b->ty);
-    if (px) return launch_batch_patches(b->ns, px, tab, b->d_tiles, b->ntiles, b->d_counters, parity, b->stream);
+    if (b->px) return launch_batch_patches(b->ns, b->px, tab, b->d_tiles, b->ntiles, b->d_counters, parity, b->stream);
     return launch_batch_step(b->ns, b->tx, tab, b->d_tiles, b->ntiles, b->d_counters, parity, b->stream);
 }
 

@@ -136,6 +136,9 @@ cudaError_t launch_step_tape_b_f32(int ns, const StepParams &p, cudaStream_t st)
 cudaError_t launch_batch_step(int ns, int tx, const StepParams *d_params, const BatchTile *d_tiles,
                               int ntiles, int *d_counters, int parity, cudaStream_t st);
 
+// Resident blocks of that launch on the current device, and its SMs.
+cudaError_t batch_march_blocks(int ns, int tx, int *blocks, int *sms);
+
 // The same on patches of px x 8 nodes (px = 16 or 32): d_tiles lists patches
 // and every patch is one block.
 cudaError_t launch_batch_patches(int ns, int px, const StepParams *d_params, const BatchTile *d_tiles, int ntiles,
