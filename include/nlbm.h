@@ -214,7 +214,9 @@ nlbm_status nlbm_get_tile(const nlbm_sim *s, int32_t *tx, int32_t *ty);
  * 48}, one untimed step and then steps_per_trial (>= 1) steps timed with
  * CUDA events on the simulation's stream, each trial from the state saved
  * in dev_scratch (device memory, 16-byte aligned, at least
- * nlbm_state_bytes()); keeps the fastest shape.  The result of a step does
+ * nlbm_state_bytes()); keeps the fastest shape.  ty = 0 is timed once where
+ * it is the same for every tx, and where it is not the march of one wave,
+ * that march's rows are one more ty (if above 8).  The result of a step does
  * not depend on the tile (every node is computed by the same code from the
  * same inputs), and the state and step counter are those of the call on
  * return; the trial launches count in nlbm_kernel_launches().  With 16-bit

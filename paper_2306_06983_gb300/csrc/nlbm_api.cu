@@ -7,6 +7,7 @@
 #include <cstdint>
 #include <cstring>
 #include <algorithm>
+#include <iterator>
 #include <new>
 #include <vector>
 
@@ -607,41 +608,58 @@ nlbm_status nlbm_autotune(nlbm_sim *s, void *dev_scratch, size_t scratch_bytes, 
         if (e0) cudaEventDestroy(e0);
         return cuda_fail(s, e, "timing events");
     }
+    // Trials: for every width that the lattice can fill (strips of tx - 4
+    // columns) the explicit rows and the library's own choice, ty = 0, which
+    // only a one-wave march makes depend on tx; where it is another form, the
+    // one-wave march is tried by its rows.  16-bit storage has one shape.
     static const int kTx[] = {64, 128, 256};
-    static const int kTy[] = {0, 8, 12, 16, 20, 24, 32, 48};
-    float best = 1e30f;
-    if (s->half()) s->ty = 0;
-    int btx = s->tx, bty = s->ty;
+    static const int kTy[] = {8, 12, 16, 20, 24, 32, 48};
+    struct Trial { int tx, ty; } trials[3 * 9];
+    int count = 0;
+    bool seen[3] = {false, false, false};
+    if (s->half()) {
+        s->ty = 0;
+        trials[count++] = Trial{s->tx, 0};
+    }
     for (int tx : kTx) {
-        // a strip of tx - 4 columns; skip widths the lattice cannot fill
-        if (!s->half() && tx > 64 && (tx / 2 - 4) >= s->kp.nx) continue;
-        for (int ty : kTy) {
-            if (s->half() && (tx != btx || ty != bty)) continue;   // 16-bit storage has one shape: timed once
-            s->tx = tx;
-            s->ty = ty;
-            for (int k = 0; k <= steps_per_trial && st == NLBM_OK; ++k) {
-                if (k == 1 && (e = cudaEventRecord(e0, s->stream)) != cudaSuccess) st = cuda_fail(s, e, "event");
-                StepParams kp = step_params(s, s->cur, s->cur ^ 1);
-                if (!s->half()) kp.pout = nullptr;
-                if (st == NLBM_OK && (e = launch_step(s, kp)) != cudaSuccess) st = cuda_fail(s, e, "trial step");
-                s->launches++;
-                s->cur ^= 1;
-            }
-            float ms = 0.f;
-            if (st == NLBM_OK &&
-                ((e = cudaEventRecord(e1, s->stream)) != cudaSuccess || (e = cudaEventSynchronize(e1)) != cudaSuccess ||
-                 (e = cudaEventElapsedTime(&ms, e0, e1)) != cudaSuccess))
-                st = cuda_fail(s, e, "trial timing");
-            if (st != NLBM_OK) break;
-            ms /= steps_per_trial;
-            if (ms < best) {
-                best = ms;
-                btx = tx;
-                bty = ty;
-            }
-            if ((st = nlbm_restore(s, dev_scratch)) != NLBM_OK) break;
+        if (s->half() || (tx > 64 && (tx / 2 - 4) >= s->kp.nx)) continue;
+        StepForm form;
+        int rows = 0;
+        const StepParams kp = step_params(s, s->cur, s->cur ^ 1);
+        e = (s->model == NLBM_MODEL_A ? step_form_a_f32 : step_form_b_f32)(s->ns, kp, tx, &form, &rows);
+        if (e != cudaSuccess) { st = cuda_fail(s, e, "trial shapes"); break; }
+        if (form == StepForm::OneWave || !seen[(int)form]) trials[count++] = Trial{tx, 0};
+        seen[(int)form] = true;
+        for (int ty : kTy) trials[count++] = Trial{tx, ty};
+        if (form != StepForm::OneWave && rows > kTy[0] && std::find(std::begin(kTy), std::end(kTy), rows) == std::end(kTy))
+            trials[count++] = Trial{tx, rows};
+    }
+    float best = 1e30f;
+    int btx = s->tx, bty = s->ty;
+    for (int i = 0; i < count && st == NLBM_OK; ++i) {
+        s->tx = trials[i].tx;
+        s->ty = trials[i].ty;
+        for (int k = 0; k <= steps_per_trial && st == NLBM_OK; ++k) {
+            if (k == 1 && (e = cudaEventRecord(e0, s->stream)) != cudaSuccess) st = cuda_fail(s, e, "event");
+            StepParams kp = step_params(s, s->cur, s->cur ^ 1);
+            if (!s->half()) kp.pout = nullptr;
+            if (st == NLBM_OK && (e = launch_step(s, kp)) != cudaSuccess) st = cuda_fail(s, e, "trial step");
+            s->launches++;
+            s->cur ^= 1;
         }
+        float ms = 0.f;
+        if (st == NLBM_OK &&
+            ((e = cudaEventRecord(e1, s->stream)) != cudaSuccess || (e = cudaEventSynchronize(e1)) != cudaSuccess ||
+             (e = cudaEventElapsedTime(&ms, e0, e1)) != cudaSuccess))
+            st = cuda_fail(s, e, "trial timing");
         if (st != NLBM_OK) break;
+        ms /= steps_per_trial;
+        if (ms < best) {
+            best = ms;
+            btx = s->tx;
+            bty = s->ty;
+        }
+        st = nlbm_restore(s, dev_scratch);
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
@@ -747,14 +765,6 @@ nlbm_status batch_fail(nlbm_batch *b, cudaError_t e, const char *what)
 {
     set_err(b->err, "%s: %s", what, cudaGetErrorString(e));
     return NLBM_ECUDA;
-}
-
-// Whether the pulls of a member's march are staged as row windows: the same
-// condition as the single-simulation launcher's.
-bool row_windows(const StepParams &kp)
-{
-    return !kp.wall_x && kp.nx % 4 == 0 &&
-           ((reinterpret_cast<uintptr_t>(kp.fin) | reinterpret_cast<uintptr_t>(kp.gin)) & 15) == 0;
 }
 
 // Tiles for the current tx and ty: px > 0 patches of px columns and 8 rows,

@@ -75,6 +75,18 @@ struct StepParams {
     float wetc[2][kMaxPhases][kMaxPhases];   // (4/eps) cos theta_pq, walls y = 0 and y = ny - 1
 };
 
+// Whether a march stages its pulls as row windows: they need nx a multiple of
+// 4 (rows and planes start on 16-byte boundaries), 16-byte aligned arrays and
+// no wall across x (a wall bounces single columns back, which a window cannot
+// express); they are used whenever they apply, even where their larger shared
+// memory leaves fewer blocks resident (N = 7: two blocks per SM with windows
+// against three with per-node pulls, and the windows are faster).
+inline bool row_windows(const StepParams &p)
+{
+    const uintptr_t a = reinterpret_cast<uintptr_t>(p.fin) | reinterpret_cast<uintptr_t>(p.gin);
+    return !p.wall_x && p.nx % 4 == 0 && (a & 15) == 0;
+}
+
 // Programmatic dependent launch (the step kernels, the ensemble kernels, the
 // adjoint's reverse passes, the initial state and the export): a kernel launched with launch_pdl is scheduled
 // as the blocks of its
@@ -121,6 +133,12 @@ cudaError_t launch_step_a_bf16(int ns, const StepParams &p, int tx, int ty, cuda
 cudaError_t launch_step_b_bf16(int ns, const StepParams &p, int tx, int ty, cudaStream_t st);
 cudaError_t launch_step_a_f16(int ns, const StepParams &p, int tx, int ty, cudaStream_t st);
 cudaError_t launch_step_b_f16(int ns, const StepParams &p, int tx, int ty, cudaStream_t st);
+
+// What an FP32 step with tx threads runs as when no rows are given, and the
+// rows of a chunk of its one-wave march (step_kernel.cuh).
+enum class StepForm { Patches, OneWave, NarrowChunks };
+cudaError_t step_form_a_f32(int ns, const StepParams &p, int tx, StepForm *form, int *wave_rows);
+cudaError_t step_form_b_f32(int ns, const StepParams &p, int tx, StepForm *form, int *wave_rows);
 
 // The FP32 step (128-thread blocks) that also writes the step's
 // intermediate fields for the adjoint to p.tape, 8 (N-1) + 13 planes in the

@@ -8,4 +8,9 @@ cudaError_t launch_step_a_f32(int ns, const StepParams &p, int tx, int ty, cudaS
     return launch_step_model<0, 0>(ns, p, tx, ty, st);
 }
 
+cudaError_t step_form_a_f32(int ns, const StepParams &p, int tx, StepForm *form, int *wave_rows)
+{
+    return step_form<0>(ns, p, tx, form, wave_rows);
+}
+
 }  // namespace nlbm

@@ -1425,40 +1425,80 @@ cudaError_t launch_step_variant(const StepParams &p, int ty, int nslots, cudaStr
 
 namespace nlbm {
 
-// Row windows need nx a multiple of 4 (rows and planes start on 16-byte
-// boundaries), 16-byte aligned arrays and no wall across x (a wall bounces
-// single columns back, which a window cannot express); they are used whenever
-// they apply, even where their larger shared memory leaves fewer blocks
-// resident (N = 7: two blocks per SM with windows against three with per-node
-// pulls, and the windows are faster).
-template <int NS, int MODEL, int T, bool TAPE = false>
-cudaError_t launch_step_f32(const StepParams &p, int ty, cudaStream_t st)
+// Resident blocks of the march's variant for p.
+template <int NS, int MODEL, int T, bool TAPE>
+cudaError_t march_slots(const StepParams &p, int *slots)
 {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    const uintptr_t a = reinterpret_cast<uintptr_t>(p.fin) | reinterpret_cast<uintptr_t>(p.gin);
-    const bool vec = !p.wall_x && p.nx % 4 == 0 && (a & 15) == 0;
+    return row_windows(p) ? variant_slots<NS, MODEL, T, true, TAPE>(dev, slots)
+                          : variant_slots<NS, MODEL, T, false, TAPE>(dev, slots);
+}
+
+// What a step without an explicit number of rows runs as: patches, a march
+// of one wave, or (long marches at N = 5 and 6) many short chunks of narrow
+// strips, which start their rows at different times where one wave marches in
+// step (us a step, one wave / 20 rows of 60 columns: 2048^2 N = 5 340 / 331, N =
+// 6 442 / 415, 1792^2 267 / 256 and 335 / 319; equal at 44 rows a chunk, slower
+// below, and slower at N = 7 and 8 on some sizes: 2304^2 N = 8 774 / 803).
+template <int NS, int MODEL, bool TAPE>
+StepForm auto_form(const StepParams &p, int T, int slots)
+{
+    const bool windows = row_windows(p);
+    const int chunks = march_chunks(p, T, slots);
+    if (use_patches<NS, MODEL>(p.ny, chunks, windows)) return StepForm::Patches;
+    if (!TAPE && (NS == 4 || NS == 5) && windows && p.ny > 50 * chunks) return StepForm::NarrowChunks;
+    return StepForm::OneWave;
+}
+
+template <int NS, int MODEL, int T, bool TAPE = false>
+cudaError_t launch_step_f32(const StepParams &p, int ty, cudaStream_t st)
+{
     int slots = 0;
-    e = vec ? variant_slots<NS, MODEL, T, true, TAPE>(dev, &slots)
-            : variant_slots<NS, MODEL, T, false, TAPE>(dev, &slots);
+    const cudaError_t e = march_slots<NS, MODEL, T, TAPE>(p, &slots);
     if (e != cudaSuccess) return e;
-    if (ty <= 0 && use_patches<NS, MODEL>(p.ny, march_chunks(p, T, slots), vec))
-        return launch_patches<NS, MODEL, 0, TAPE>(p, st);
-    // Long marches at N = 5 and 6: many short chunks of narrow strips start
-    // their rows at different times where one wave marches in step (us a step,
-    // one wave / 20 rows of 60 columns: 2048^2 N = 5 340 / 331, N = 6 442 / 415,
-    // 1792^2 267 / 256 and 335 / 319; equal at 44 rows a chunk, slower below,
-    // and slower at N = 7 and 8 on some sizes: 2304^2 N = 8 774 / 803).
+    const StepForm form = ty > 0 ? StepForm::OneWave : auto_form<NS, MODEL, TAPE>(p, T, slots);
+    if (form == StepForm::Patches) return launch_patches<NS, MODEL, 0, TAPE>(p, st);
     if constexpr (!TAPE && (NS == 4 || NS == 5)) {
-        if (ty <= 0 && vec && p.ny > 50 * march_chunks(p, T, slots)) {
-            if ((e = variant_slots<NS, MODEL, 64, true, TAPE>(dev, &slots)) != cudaSuccess) return e;
-            return launch_step_variant<NS, MODEL, 64, true, TAPE>(p, 20, slots, st);
+        if (form == StepForm::NarrowChunks) {
+            int narrow = 0;
+            const cudaError_t en = march_slots<NS, MODEL, 64, TAPE>(p, &narrow);
+            return en != cudaSuccess ? en : launch_step_variant<NS, MODEL, 64, true, TAPE>(p, 20, narrow, st);
         }
     }
-    return vec ? launch_step_variant<NS, MODEL, T, true, TAPE>(p, ty, slots, st)
-               : launch_step_variant<NS, MODEL, T, false, TAPE>(p, ty, slots, st);
+    return row_windows(p) ? launch_step_variant<NS, MODEL, T, true, TAPE>(p, ty, slots, st)
+                          : launch_step_variant<NS, MODEL, T, false, TAPE>(p, ty, slots, st);
+}
+
+// The form of a step with tx threads and no explicit rows, and the rows of
+// a chunk of its one-wave march (FP32 storage).
+template <int NS, int MODEL, int T>
+cudaError_t step_form_nt(const StepParams &p, StepForm *form, int *wave_rows)
+{
+    int slots = 0;
+    const cudaError_t e = march_slots<NS, MODEL, T, false>(p, &slots);
+    if (e != cudaSuccess) return e;
+    const int chunks = march_chunks(p, T, slots);
+    *form = auto_form<NS, MODEL, false>(p, T, slots);
+    *wave_rows = (p.ny + chunks - 1) / chunks;
+    return cudaSuccess;
+}
+template <int MODEL>
+cudaError_t step_form(int ns, const StepParams &p, int tx, StepForm *form, int *wave_rows)
+{
+    switch (ns) {
+#define NLBM_CASE(K)                                                                             \
+    case K:                                                                                      \
+        return tx == 64    ? step_form_nt<K, MODEL, 64>(p, form, wave_rows)                      \
+               : tx == 128 ? step_form_nt<K, MODEL, 128>(p, form, wave_rows)                     \
+               : tx == 256 ? step_form_nt<K, MODEL, 256>(p, form, wave_rows)                     \
+                           : cudaErrorInvalidValue;
+        NLBM_CASE(1) NLBM_CASE(2) NLBM_CASE(3) NLBM_CASE(4) NLBM_CASE(5) NLBM_CASE(6) NLBM_CASE(7)
+#undef NLBM_CASE
+    default: return cudaErrorInvalidValue;
+    }
 }
 
 template <int NS, int MODEL, int ST>
