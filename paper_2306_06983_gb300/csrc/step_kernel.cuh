@@ -1437,20 +1437,43 @@ cudaError_t march_slots(const StepParams &p, int *slots)
                           : variant_slots<NS, MODEL, T, false, TAPE>(dev, slots);
 }
 
+// Nodes that a march of T-thread blocks in `chunks` row chunks updates, its
+// strips padded to T - 4 columns, with 3/4 row more a chunk (the cost of its 6
+// extra rows, mostly in L2; 1/4 row for Model A at N = 8, fitted like the gain
+// of use_patches).
+template <int NS, int MODEL>
+inline double march_nodes(const StepParams &p, int T, int chunks)
+{
+    constexpr double kRows = NS == 7 && MODEL == 0 ? .25 : .75;
+    return (double)((p.nx + T - 5) / (T - 4)) * (T - 4) * (p.ny + kRows * chunks);
+}
+
 // What a step without an explicit number of rows runs as: patches, a march
-// of one wave, or (long marches at N = 5 and 6) many short chunks of narrow
+// of one wave, or (N = 6, Model B at N = 5) many 20-row chunks of narrow
 // strips, which start their rows at different times where one wave marches in
-// step (us a step, one wave / 20 rows of 60 columns: 2048^2 N = 5 340 / 331, N =
-// 6 442 / 415, 1792^2 267 / 256 and 335 / 319; equal at 44 rows a chunk, slower
-// below, and slower at N = 7 and 8 on some sizes: 2304^2 N = 8 774 / 803).
+// step.  Those gain from 50 rows a chunk of the wave on (us a step, one wave /
+// 20 rows of 60 columns, N = 5: 2048^2 340 / 331, 1792^2 267 / 256; equal at 44
+// rows); at N = 6, with two blocks an SM, where their strips waste less than
+// they lose on short chunks (2048^2 442 / 415, 1500^2 244 / 235, 1792^2 334 / 319,
+// but 1408^2 214 / 217, 1472^2 222 / 231, 1600^2 262 / 269).  At N = 7 and 8 they
+// lose on some sizes (2304^2 N = 8 774 / 803), and for Model A at N = 5 to patches
+// (2048^2 331 / 327).
 template <int NS, int MODEL, bool TAPE>
 StepForm auto_form(const StepParams &p, int T, int slots)
 {
     const bool windows = row_windows(p);
     const int chunks = march_chunks(p, T, slots);
-    if (use_patches<NS, MODEL>(p.ny, chunks, windows)) return StepForm::Patches;
-    if (!TAPE && (NS == 4 || NS == 5) && windows && p.ny > 50 * chunks) return StepForm::NarrowChunks;
-    return StepForm::OneWave;
+    StepForm form = StepForm::OneWave;
+    double nodes = march_nodes<NS, MODEL>(p, T, chunks);
+    if (!TAPE && (NS == 5 || (NS == 4 && MODEL == 1)) && windows && p.ny > 50 * chunks) {
+        const double rate = NS == 4 ? 1. : p.ny > 85 * chunks ? .98 : p.ny > 60 * chunks ? 1.02 : 1.04;
+        const double narrow = rate * march_nodes<NS, MODEL>(p, 64, chunks);
+        if (narrow < nodes) {
+            form = StepForm::NarrowChunks;
+            nodes = narrow;
+        }
+    }
+    return use_patches<NS, MODEL>(p, nodes, windows) ? StepForm::Patches : form;
 }
 
 template <int NS, int MODEL, int T, bool TAPE = false>

@@ -288,23 +288,22 @@ cudaError_t launch_patches(const StepParams &p, cudaStream_t st)
     return launch_patch_variant<NS, MODEL, ST, 16, 8, kNarrowMin, TAPE>(p, st);
 }
 
-// Whether an FP32 step runs on patches rather than as a march of `chunks` row
-// chunks; windows: the march would stage row windows.  A march costs 6 extra
-// rows a chunk, a patch 0.7 to 0.9 extra pulls and a third of the sources per
-// node (us a step, march / patches, rows a chunk; Model B: 64^2 N = 3 6.4 /
-// 3.5, 2 rows; 256^2 N = 5 15.7 / 8.0, 2; 512^2 N = 5 32.0 / 24.8, 6, N = 8 56.4
-// / 52.0, 8; 1024^2 N = 5 94.2 / 91.5, 20, N = 7 141.6 / 140.8, 31; 2048^2 N = 5
-// 340 / 366, 78, N = 8 651 / 683).  Ahead at every size: N = 3 (2048^2 200 /
-// 192), Model A at N = 5 (339 / 330) and N = 8 (634 / 599, 1024^2 172 / 158);
-// and, where patches are wide, lattices that march without row windows (1021^2
-// N = 8 210 / 185, 2045^2 N = 3 221 / 209, N = 8 761 / 700; narrow patches lose
-// there at size, N = 5 380 / 454).  N = 2, with the least work to repeat a
-// row, turns at fewer rows (1021^2, 10 rows: 43 / 46; 512^2, 3: 16.4 / 10.4).
+// Whether an FP32 step runs on patches rather than as a march that updates
+// march_nodes nodes (see there): a march spends `gain` of a patch's time on a
+// node.  The gain was fitted to both forms of 38 lattices (256 x 1024 to
+// 1920^2) per phase count and model; it picks the slower one by 1.3 % at most
+// on them (us a step, march / patches, Model B where not said: 256^2 N = 5
+// 15.7 / 8.0; 768^2 N = 7 77 / 85, N = 2 24.6 / 21.8; 832^2 N = 8 115 / 123; 1100^2
+// N = 5 101 / 108, N = 4 79 / 83; 1024^2 N = 6 Model A 118 / 112; 256 x 4096 N = 5
+// 114 / 91; 1472^2 N = 6 222 / 243).  1: patches at every size (2048^2 N = 3 200 /
+// 192); so it is for most lattices without row windows (1279^2 N = 6 234 / 203,
+// 2045^2 N = 8 761 / 700).
 template <int NS, int MODEL>
-inline bool use_patches(int ny, int chunks, bool windows)
+inline bool use_patches(const StepParams &p, double march_nodes, bool windows)
 {
-    if (NS == 2 || (MODEL == 0 && (NS == 4 || NS == 7)) || (!windows && NS > 1 && wide_patches<NS, MODEL, 0>())) return true;
-    return ny <= (NS == 1 ? 8 : 24) * chunks;
+    constexpr double kGain[2][7] = {{.865, 1., .905, .965, .93, .88, .9725}, {.865, 1., .905, .895, .92, .88, .82}};
+    const double gain = windows ? kGain[MODEL][NS - 1] : NS == 1 ? .835 : NS == 4 && MODEL == 1 ? .90 : 1.;
+    return gain * march_nodes >= (double)p.nx * p.ny;
 }
 
 }  // namespace nlbm

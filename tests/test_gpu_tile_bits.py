@@ -31,8 +31,9 @@ def state(p, phi0, tile, steps=5):
     return out
 
 
-# rows that are staged as windows and rows that are not; walls
-LATTICES = [(96, 72, False, False), (67, 45, True, True), (130, 41, False, True)]
+# rows that are staged as windows and rows that are not; walls; patches of
+# either width
+LATTICES = [(96, 72, False, False), (67, 45, True, True), (130, 41, False, True), (512, 128, False, False)]
 
 
 @pytest.mark.parametrize("model,n", [("B", 1.0), ("A", 1.0), ("A", 1.5), ("A", 3.0), ("A", 6.0)])
@@ -48,13 +49,14 @@ def test_small_lattices(N, model, n):
             assert torch.equal(a, state(p, phi0, tile)), (nx, ny, tile)
 
 
-@pytest.mark.parametrize("nx", [2048, 2046])
-@pytest.mark.parametrize("N,model", [(5, "B"), (6, "A"), (6, "B")])
-def test_long_marches(N, model, nx):
-    """Lattices of more than 50 rows a chunk (strips of 60 columns and 20
-    rows where rows are staged as windows)."""
+@pytest.mark.parametrize("N,model,nx,ny", [
+    (5, "B", 2048, 1472), (6, "A", 2048, 1472), (6, "B", 2048, 1472), (5, "B", 2046, 1472), (6, "B", 2046, 1472),
+    (7, "A", 840, 832), (8, "B", 744, 704), (4, "B", 1116, 1088), (2, "A", 1240, 960)])
+def test_marches_and_patches_at_size(N, model, nx, ny):
+    """Lattices that the library marches by itself: one wave, or (N = 5 and 6,
+    over 50 rows a chunk) strips of 60 columns and 20 rows; at 2046 columns
+    rows are not staged as windows."""
     import torch
-    ny = 1472
     p, phi0 = W.random_smooth(64, 64, N, seed=N, model=model, n_disks=4)
     phi0 = torch.from_numpy(phi0.astype(np.float32)).cuda().repeat(1, ny // 64, nx // 64 + 1)[:, :, :nx].contiguous()
     p = dict(p, nx=nx, ny=ny)
