@@ -605,25 +605,28 @@ __device__ __forceinline__ float inv_norm2(float n2, float delta2)
 
 // Model A weight max(phi, 0)^n, integer n by multiplication from the left.  n
 // = 1 and 2 leave before the longer chain, which has no loop (us a step, loop /
-// one chain of predicated products / this: 2048^2 N = 6 n = 1 427 / 420 / 408, n
-// = 3 465 / 420 / 414, n = 6 480 / 434 / 414; 1500^2 N = 6 n = 1 235 / 239 / 232, N =
-// 3 n = 1 113.0 / 114.0 / 113.2), but for N >= 7, where the longer chain costs
-// registers that are not there (1024^2 N = 8, n = 1: 158 -> 165).
+// one chain of predicated products / this: 2048^2 N = 6 n = 1 427 / 420 / 405, n
+// = 6 480 / 434 / 421, N = 5 n = 1 341 / 335 / 327; 1500^2 N = 6 n = 1 235 / 239 /
+// 231, N = 3 n = 1 113.0 / 114.0 / 113.2), by a branch of their own at N = 6
+// (1024^2 n = 1 120.5 -> 117.6).  At N >= 7 the longer chain costs registers that
+// are not there (1024^2 N = 8, n = 1: 158 -> 165).
 template <int NS>
 __device__ __forceinline__ float model_a_weight(const StepParams &P, float ph)
 {
     const float pc = fmaxf(ph, 0.f);
-    if constexpr (NS >= 6) {
+    if constexpr (NS >= 5) {
         if (P.model_n_int == 1) return pc;
         if (P.model_n_int == 2) return pc * pc;
+    }
+    if constexpr (NS >= 6) {
         if (P.model_n_int > 2) {
             float wq = pc;
             for (int k = 1; k < P.model_n_int; ++k) wq *= pc;
             return wq;
         }
-    } else if (P.model_n_int > 0) {   // at most 8
-        float wq = P.model_n_int > 1 ? pc * pc : pc;
-        if (P.model_n_int > 2) {
+    } else if (P.model_n_int > (NS == 5 ? 2 : 0)) {   // at most 8
+        float wq = NS == 5 || P.model_n_int > 1 ? pc * pc : pc;
+        if (NS == 5 || P.model_n_int > 2) {
             wq *= pc;
             if (P.model_n_int > 3) wq *= pc;
             if (P.model_n_int > 4) wq *= pc;
