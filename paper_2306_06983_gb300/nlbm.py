@@ -717,6 +717,19 @@ def pair_list(N: int):
     return [(p, q) for p in range(N) for q in range(p + 1, N)]
 
 
+def _final_phi(params: dict, phi0, nsteps: int):
+    """phi(T) [N, ny, nx] of a plain run on phi0's device."""
+    import torch
+    sim = Simulation(params, device=phi0.device)
+    t = phi0.to(device=sim.device, dtype=torch.float32).contiguous()
+    out = torch.empty((sim.N, sim.ny, sim.nx), dtype=torch.float32, device=sim.device)
+    nlbm_set_phi(sim.h, t.data_ptr())
+    sim.step(nsteps)
+    nlbm_get_moments(sim.h, ctypes.c_void_p(out.data_ptr()))
+    sim.close()
+    return out
+
+
 def _make_function():
     import torch
 
@@ -727,12 +740,17 @@ def _make_function():
         (1,2), (1,3), ..., (N-1,N); mobility: 0-d tensor."""
 
         @staticmethod
-        def forward(ctx, phi0, sigma_pairs, mobility, params, nsteps, every):
+        def forward(ctx, phi0, sigma_pairs, mobility, params, nsteps, every, sweep=True):
             N = int(params["n_phases"])
             sig = np.zeros((N, N))
             for (p, q), v in zip(pair_list(N), sigma_pairs.detach().cpu().double().tolist()):
                 sig[p, q] = sig[q, p] = v
             q = dict(params, sigma=sig.tolist(), mobility=float(mobility.detach().cpu()))
+            if not sweep:
+                # no gradient will be asked for: a plain run, without
+                # checkpoints and tapes, of what a differentiable one takes
+                nlbm_adjoint_workspace_bytes(q, nsteps, every)
+                return _final_phi(q, phi0.detach(), nsteps)
             run = AdjointRun(q, nsteps, every, device=phi0.device)
             out = run.forward(phi0.detach())
             ctx.run = run
@@ -754,7 +772,7 @@ def _make_function():
             gpairs = torch.tensor([gs[p, q] for p, q in pair_list(N)], dtype=ctx.sdtype)
             ctx.run.close()
             ctx.run = None
-            return g0, gpairs, torch.tensor(gm, dtype=ctx.sdtype), None, None, None
+            return g0, gpairs, torch.tensor(gm, dtype=ctx.sdtype), None, None, None, None
 
     return NPhaseLBM
 
@@ -767,4 +785,6 @@ def nphase_lbm(phi0, sigma_pairs, mobility, params: dict, nsteps: int, every: in
     global _FN
     if _FN is None:
         _FN = _make_function()
-    return _FN.apply(phi0, sigma_pairs, mobility, params, nsteps, every)
+    import torch
+    sweep = torch.is_grad_enabled() and any(t.requires_grad for t in (phi0, sigma_pairs, mobility))
+    return _FN.apply(phi0, sigma_pairs, mobility, params, nsteps, every, sweep)
