@@ -385,9 +385,9 @@ nlbm_status nlbm_adjoint_forward(nlbm_adjoint *a, const float *dev_phi0, float *
  * *host_grad_mobility (may be NULL).  The sweep is the same launch sequence
  * after every forward of a handle: on a stream other than the legacy default
  * one, the first call captures it into a CUDA graph (kernel loading and
- * capture take a while once) and later calls replay it; another sweep after
- * the same forward rebuilds the last segment as well, without the graph.
- * Synchronizes. */
+ * capture take a while once) and later calls replay it; another sweep of the
+ * same forward rebuilds the last segment as well; the second such call
+ * captures that sequence into a graph of its own.  Synchronizes. */
 nlbm_status nlbm_adjoint_backward(nlbm_adjoint *a, const float *dev_seed, float *dev_grad_phi0,
                                   double *host_grad_sigma, double *host_grad_mobility);
 
