@@ -372,7 +372,8 @@ nlbm_status nlbm_adjoint_create(const nlbm_params *p, int32_t nsteps, int32_t ch
                                 nlbm_adjoint **out);
 
 /* Run the nsteps forward steps from dev_phi0 [N-1][ny][nx] (as
- * nlbm_set_phi()), storing the checkpoints and the last segment's tapes (the
+ * nlbm_set_phi()), storing the checkpoints and, unless the three forwards
+ * before it were not followed by a sweep, the last segment's tapes (the
  * reverse sweep starts from them); write phi(T) [N][ny][nx] into
  * dev_phi_final if non-NULL.  Asynchronous. */
 nlbm_status nlbm_adjoint_forward(nlbm_adjoint *a, const float *dev_phi0, float *dev_phi_final);
@@ -383,11 +384,12 @@ nlbm_status nlbm_adjoint_forward(nlbm_adjoint *a, const float *dev_phi0, float *
  * host_grad_sigma [N*N] (symmetric: entry (p, q) is the derivative with
  * respect to the pair's single value; may be NULL) and dL/dM into
  * *host_grad_mobility (may be NULL).  The sweep is the same launch sequence
- * after every forward of a handle: on a stream other than the legacy default
+ * after every forward that taped: on a stream other than the legacy default
  * one, the first call captures it into a CUDA graph (kernel loading and
- * capture take a while once) and later calls replay it; another sweep of the
- * same forward rebuilds the last segment as well; the second such call
- * captures that sequence into a graph of its own.  Synchronizes. */
+ * capture take a while once) and later calls replay it.  After other forwards,
+ * and for another sweep of the same forward, it rebuilds the last segment as
+ * well; the second such call captures that sequence into a graph of its own.
+ * Synchronizes. */
 nlbm_status nlbm_adjoint_backward(nlbm_adjoint *a, const float *dev_seed, float *dev_grad_phi0,
                                   double *host_grad_sigma, double *host_grad_mobility);
 

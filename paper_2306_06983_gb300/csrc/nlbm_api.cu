@@ -1196,6 +1196,7 @@ struct nlbm_adjoint {
     float *seed_buf;           // [N][plane] copy of the caller's dL/dphi(T)
     float *grad_buf;           // [N-1][plane] dL/dphi_0
     int taped;                 // segment whose states and tapes seg / tapes hold, -1: none
+    int unswept;               // forwards since the last sweep, counted to kUnswept
     // the whole reverse sweep as a graph: [0] from the last segment's tapes
     // that forward kept, captured on first use; [1] rebuilding them, captured
     // on second use (a handle often needs that sweep once or never)
@@ -1206,6 +1207,8 @@ struct nlbm_adjoint {
 };
 
 namespace {
+
+constexpr int kUnswept = 3;   // see nlbm_adjoint_forward()
 
 // State of a simulation between steps: f [9 NS], g [8], u [2], phi [NS],
 // m_phi [2] planes (FP32 storage).
@@ -1312,6 +1315,22 @@ float *adj_segment_state(const nlbm_adjoint *a, int k, int s)
 int adj_segment_length(const nlbm_adjoint *a, int k)
 {
     return (k + 1) * a->every <= a->nsteps ? a->every : a->nsteps - k * a->every;
+}
+
+// `steps` steps from checkpoint k without tapes, through the first two slots
+// of the segment's states or, the last one, into `end` if given; returns
+// where that one was written.
+cudaError_t adj_run_segment(nlbm_adjoint *a, int k, int steps, float *end, const float **last)
+{
+    const float *in = a->ckpt + a->state_floats * k;
+    for (int t = 0; t < steps; ++t) {
+        float *out = end && t + 1 == steps ? end : a->seg + a->state_floats * (t & 1);
+        const cudaError_t e = adj_step(a, in, out, nullptr);
+        if (e != cudaSuccess) return e;
+        in = out;
+    }
+    *last = in;
+    return cudaSuccess;
 }
 
 // The states and tapes of segment k from its checkpoint: one taping step
@@ -1505,6 +1524,7 @@ nlbm_status nlbm_adjoint_create(const nlbm_params *p, int32_t nsteps, int32_t ch
     a->partials = (double *)(ws + L.partials);
     a->acc = (double *)(ws + L.acc);
     a->taped = -1;
+    a->unswept = 0;
     a->forward_done = false;
     a->err[0] = 0;
     *out = a;
@@ -1518,7 +1538,11 @@ nlbm_status nlbm_adjoint_forward(nlbm_adjoint *a, const float *dev_phi0, float *
     // The initial state is written as the first checkpoint; from there on a
     // step reads one packed record and writes the next, every segment's last
     // step straight into the next checkpoint.  The last segment runs the
-    // taping kernel: its states and tapes are the first that a sweep needs.
+    // taping kernel, as its states and tapes are the first that a sweep needs,
+    // until kUnswept forwards in a row were not followed by one.  Taping every
+    // step costs a forward 25 to 40 % (1024^2, us a step: N = 2 42 -> 60, N = 3
+    // 55 -> 76, N = 5 96 -> 121) and saves the sweep as much as the taped
+    // forward takes, so that a few of them unread (a line search) still pay.
     const size_t pl = a->plane;
     const int ns = a->ns, last = a->nckpt - 1;
     StepParams kp = adj_params_from_state(a, a->ckpt);
@@ -1536,19 +1560,21 @@ nlbm_status nlbm_adjoint_forward(nlbm_adjoint *a, const float *dev_phi0, float *
     s->launches++;
     a->forward_done = false;
     a->taped = -1;
-    for (int k = 0; k < last; ++k) {
-        const float *in = a->ckpt + a->state_floats * k;
-        for (int t = 0; t < a->every; ++t) {
-            float *out = t + 1 < a->every ? a->seg + a->state_floats * (t & 1) : a->ckpt + a->state_floats * (k + 1);
-            if ((e = adj_step(a, in, out, nullptr)) != cudaSuccess) return adj_fail(a, e, "forward step");
-            in = out;
-        }
+    const bool tape = a->unswept < kUnswept;
+    a->unswept += tape;
+    const float *end;
+    for (int k = 0; k < last; ++k)
+        if ((e = adj_run_segment(a, k, a->every, a->ckpt + a->state_floats * (k + 1), &end)) != cudaSuccess)
+            return adj_fail(a, e, "forward step");
+    const int len = adj_segment_length(a, last);
+    e = tape ? adj_tape_segment(a, last) : adj_run_segment(a, last, len, nullptr, &end);
+    if (e != cudaSuccess) return adj_fail(a, e, "forward step");
+    if (tape) {
+        end = a->seg + a->state_floats * len;
+        a->taped = last;
     }
-    if ((e = adj_tape_segment(a, last)) != cudaSuccess) return adj_fail(a, e, "forward step");
     s->launches += a->nsteps;
-    a->taped = last;
     if (dev_phi_final) {
-        const float *end = a->seg + a->state_floats * adj_segment_length(a, last);
         e = launch_export(ns, end + pl * (9 * ns + 10), nullptr, nullptr, (unsigned)pl, dev_phi_final, nullptr, nullptr,
                           a->stream);
         if (e != cudaSuccess) return adj_fail(a, e, "export kernel");
@@ -1568,10 +1594,11 @@ nlbm_status nlbm_adjoint_backward(nlbm_adjoint *a, const float *dev_seed, float 
     const AdjCounts c = adj_counts(ns);
     cudaError_t e = cudaMemcpyAsync(a->seed_buf, dev_seed, pb * N, cudaMemcpyDeviceToDevice, a->stream);
     if (e != cudaSuccess) return adj_fail(a, e, "seed copy");
-    // After a forward, and for another sweep of the same forward, the sweep is
-    // one sequence of launches each on every call of this handle: captured
-    // into a CUDA graph (on a capturable stream) and replayed (256^2 N = 3,
-    // another sweep of 20 steps, launched / replayed: 26.2 / 24.8 us a step).
+    // After a forward that taped, and after one that did not or for another
+    // sweep of the same forward, the sweep is one sequence of launches each
+    // on every call of this handle: captured into a CUDA graph (on a
+    // capturable stream) and replayed (256^2 N = 3, another sweep of 20 steps,
+    // launched / replayed: 26.2 / 24.8 us a step).
     const bool rebuild_last = a->taped != a->nckpt - 1;
     const int kind = rebuild_last ? 1 : 0;
     if (!a->graph[kind] && a->sweeps[kind] == kind && a->stream != nullptr) {
@@ -1586,6 +1613,7 @@ nlbm_status nlbm_adjoint_backward(nlbm_adjoint *a, const float *dev_seed, float 
         cudaGetLastError();   // a failed capture leaves the direct path
     }
     a->sweeps[kind] += a->sweeps[kind] <= kind;   // counted as far as it matters
+    a->unswept = 0;
     a->taped = -1;
     if (a->graph[kind]) {
         e = cudaGraphLaunch(a->graph[kind], a->stream);
