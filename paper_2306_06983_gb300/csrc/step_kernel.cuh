@@ -776,20 +776,16 @@ __device__ __forceinline__ void wet_ghost(const StepParams &P, int ra, float (&p
     for (int p = 0; p < NS; ++p) ph[p] += k2 * sp[p];
 }
 
-// What complete_node reads of its own node from the rings of the row march:
-// j and phi_lo (j rows of the node's row) and phi of a neighbour.
+// What complete_node reads of its own node from the rings of the row march: j
+// and phi_lo (j rows of the node's row).
 template <int NS>
 struct OwnRing {
-    const float *s_j, *s_phi;
-    int T, t, sm, s0, sp;
+    const float *s_j;
+    int T, t;
     static constexpr int NE = ring_even(NS);
     template <class V> __device__ __forceinline__ V jx(int p) const { return rld<V>(s_j, T, p, t); }
     template <class V> __device__ __forceinline__ V jy(int p) const { return rld<V>(s_j + NE * T, T, p, t); }
     template <class V> __device__ __forceinline__ V plo(int p) const { return rld<V>(s_j + 2 * NE * T, T, p, t); }
-    template <class V> __device__ __forceinline__ V phi_at(int p, int cx, int cy) const
-    {
-        return rld<V>(s_phi + (cy > 0 ? sp : (cy < 0 ? sm : s0)) * NE * T, T, p, t + cx);
-    }
 };
 
 // a b + c d with the first product fused.  Left to the compiler, which of the
@@ -1165,7 +1161,7 @@ __device__ __forceinline__ void step_tile(const StepParams &P, const int x0, con
     int a5 = slot5(y0 - 2), a3 = slot3(y0 - 2);
     for (int it = 0; it < TYe + 4; ++it) {
         const int ra = y0 - 2 + it;
-        const int a5m1 = a5 == 0 ? 4 : a5 - 1, a5m2 = a5 >= 2 ? a5 - 2 : a5 + 3, a5m3 = a5 >= 3 ? a5 - 3 : a5 + 2;
+        const int a5m1 = a5 == 0 ? 4 : a5 - 1, a5m2 = a5 >= 2 ? a5 - 2 : a5 + 3;
         const int a3m1 = a3 == 0 ? 2 : a3 - 1, a3m2 = a3 >= 2 ? a3 - 2 : a3 + 1;
         // stage-C inputs of row ra - 2, requested before stages A and B
         // (loaded raw; anything computed from them waits until stage C, so
@@ -1279,7 +1275,6 @@ __device__ __forceinline__ void step_tile(const StepParams &P, const int x0, con
         // ---------------------------------------------------- stage C
         if (do_c) {
             const int y = ra - 2;
-            const int sm = a5m3, s0 = a5m2, sp = a5m1;
             float ph[N], gx[N], gy[N], lap[N];
             close_phases<NS>(PHc, GXc, GYc, LPc, ph, gx, gy, lap);
 
@@ -1300,7 +1295,7 @@ __device__ __forceinline__ void step_tile(const StepParams &P, const int x0, con
                     for (int i = 1; i < 9; ++i) gv[i] = g[i];
                 }
             };
-            const OwnRing<NS> own_node{s_j + a3m2 * 3 * NE * T, s_phi, T, t, sm, s0, sp};
+            const OwnRing<NS> own_node{s_j + a3m2 * 3 * NE * T, T, t};
             complete_node<NS, 0, TAPE>(P, node, xg, y, ph, gx, gy, lap, s_w + a3 * T + t, s_w + a3m2 * T + t,
                                         s_w + a3m1 * T + t, load_g, php, mpx, mpy, Rcx, Rcy, Mcx, Mcy, Ucx, Ucy,
                                         own_node);

@@ -81,8 +81,9 @@ __device__ __forceinline__ void pull_direct(const StepParams &P, const unsigned 
     if (NS & 1) pull_direct_v<float, NS, ST, OWN>(P, idx, self, NS - 1, ph, plo, jx, jy);
 }
 
-// OwnRing's counterpart: j and phi_lo in the thread's own slots, phi in the
-// patch's ring (row of 2 ceil(NS / 2) values per column, see ring_idx).
+// OwnRing's counterpart: j and phi_lo in the thread's own slots, and phi of a
+// neighbour (16-bit storage) in the patch's ring (row of 2 ceil(NS / 2) values
+// per column, see ring_idx).
 template <int NS, int RX, int T>
 struct OwnPatch {
     const float *s_j, *s_phi;   // s_phi: the node's row
