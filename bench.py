@@ -66,14 +66,14 @@ def adjoint_bytes_per_lup(N: int, kept: float = 0.0) -> dict:
     FP32; NS = N - 1 solved phases), each field a pass reads or writes counted
     once per pass; kept: the share of the steps that are taped by the forward
     (its last segment) instead of being rebuilt in the sweep.
-    Forward step 8(10N + 2), and 8 NS + 13 tape floats where it tapes; reverse
+    Forward step 8(10N + 2), and 8 NS + 12 tape floats where it tapes; reverse
     step = the taping rebuild (a forward step that also writes the tape) and
     two passes:
     1 collision: 8 NS + 12 tape, NS + 4 state, NS + 4 seed and 3 NS + 8
       gathered floats read, 9 NS + 16 written;
     2 source and stencils: 9 NS + 10 floats read, NS + 2 written."""
     NS = N - 1
-    step, tape = 8 * (10 * N + 2), 4 * (8 * NS + 13)
+    step, tape = 8 * (10 * N + 2), 4 * (8 * NS + 12)
     fwd = step + kept * tape
     rebuild = (1.0 - kept) * (step + tape)
     collide = 4 * ((8 * NS + 12) + (NS + 4) + (NS + 4) + (3 * NS + 8) + (9 * NS + 16))

@@ -357,10 +357,10 @@ const char *nlbm_batch_last_error(const nlbm_batch *b);
 typedef struct nlbm_adjoint nlbm_adjoint;
 
 /* Device workspace bytes for nsteps >= 1 steps with a checkpoint every
- * checkpoint_every >= 1 steps: the simulation, ceil(nsteps / every)
- * checkpoints and every + 1 segment states of 10(N-1)+12 floats a node,
- * `every` tapes of the segment's steps (8(N-1)+13 floats a node), the
- * adjoint fields.  Host only. */
+ * checkpoint_every >= 1 steps: ceil(nsteps / every) checkpoints and
+ * every + 1 segment states of 10(N-1)+12 floats a node, `every` tapes of the
+ * segment's steps (8(N-1)+12 floats a node), the adjoint fields (39(N-1)+50
+ * floats a node).  Host only. */
 nlbm_status nlbm_adjoint_workspace_bytes(const nlbm_params *p, int32_t nsteps, int32_t checkpoint_every,
                                          size_t *bytes);
 

@@ -852,7 +852,7 @@ __device__ __forceinline__ void rev_pull_node(const StepParams &P, const AdjFiel
 // that the neighbours they gather from are mostly the block's own lines.
 constexpr int kRevX = 32, kRevY = 8, kRevThreads = kRevX * kRevY;
 
-inline int rev_blocks(const StepParams &P) { return ((P.nx + kRevX - 1) / kRevX) * ((P.ny + kRevY - 1) / kRevY); }
+inline int rev_blocks(int nx, int ny) { return ((nx + kRevX - 1) / kRevX) * ((ny + kRevY - 1) / kRevY); }
 
 // Adds the block's sums of K per-thread values to gacc[q][block] in FP64, in
 // a fixed order: lane l of a warp sums the values of threads l, l + 32, ...,
@@ -1004,15 +1004,16 @@ __global__ void __launch_bounds__(256) rev_pull_kernel(const StepParams P, AdjFi
 
 constexpr int kRedThreads = 256;
 
-// Fixed-order FP64 sums of K per-node fields, added to acc[K].
-__global__ void __launch_bounds__(kRedThreads) reduce_partial_kernel(const double *__restrict__ contrib, int K,
+// FP64 sums of K arrays of n values (a block's sums of a parameter's terms) in
+// a fixed order: partial sums per block of this grid, then those.
+__global__ void __launch_bounds__(kRedThreads) reduce_partial_kernel(const double *__restrict__ sums, int K,
                                                                      unsigned n, double *partials)
 {
     __shared__ double red[kRedThreads];
     for (int c = 0; c < K; ++c) {
         double v = 0.0;
         for (unsigned k = blockIdx.x * kRedThreads + threadIdx.x; k < n; k += gridDim.x * kRedThreads)
-            v += contrib[(size_t)c * n + k];
+            v += sums[(size_t)c * n + k];
         red[threadIdx.x] = v;
         __syncthreads();
         for (int s = kRedThreads / 2; s > 0; s >>= 1) {
@@ -1044,7 +1045,7 @@ int blocks_for(unsigned n)
 template <int NS, int MODEL, bool WALLS>
 cudaError_t reverse_passes(const StepParams &P, const AdjTape &T, const AdjFields &A, bool taped, cudaStream_t st)
 {
-    const int nb = rev_blocks(P);
+    const int nb = rev_blocks(P.nx, P.ny);
     cudaError_t e = taped ? launch_pdl(rev_collide_kernel<NS, true, WALLS>, nb, kRevThreads, 0, st, P, T, A)
                           : launch_pdl(rev_collide_kernel<NS, false, WALLS>, nb, kRevThreads, 0, st, P, T, A);
     if (e != cudaSuccess) return e;
@@ -1096,7 +1097,7 @@ cudaError_t launch_reverse_step(int ns, const StepParams &P, const AdjTape &T, c
     }
 }
 
-int adj_sum_blocks(const StepParams &P) { return rev_blocks(P); }
+int adj_sum_blocks(int nx, int ny) { return rev_blocks(nx, ny); }
 
 cudaError_t launch_grad_reduce(const double *gacc, int K, unsigned plane, double *partials, double *acc,
                                cudaStream_t st)

@@ -17,7 +17,7 @@ struct AdjTape {
     float *lap;    // [N-1]  lap phi_p (Eq. (27))
     float *R;      // [2(N-1)] Model B source (Eqs. (3), (4))
     float *mphi;   // [2]    m_phi (Eq. (13))
-    float *w;      // [1]    m_phi,x u_y - u_x m_phi,y (previous velocity)
+    float *w;      // [1]    m_phi,x u_y - u_x m_phi,y (previous velocity); not kept for a sweep
     float *F;      // [2]    F_s + F_c
 };
 
@@ -56,8 +56,8 @@ struct AdjFields {
 // the seeds, and a last pass writes lf_in and lg_in.
 cudaError_t launch_reverse_step(int ns, const StepParams &P, const AdjTape &T, const AdjFields &A, bool taped,
                                 cudaStream_t st);
-// Number of partial sums per parameter in gacc.
-int adj_sum_blocks(const StepParams &P);
+// Number of partial sums per parameter in gacc on an nx x ny lattice.
+int adj_sum_blocks(int nx, int ny);
 // acc[c] = sum of gacc[c][n] over n, c < K, in a fixed order (FP64).
 cudaError_t launch_grad_reduce(const double *gacc, int K, unsigned n, double *partials, double *acc,
                                cudaStream_t st);

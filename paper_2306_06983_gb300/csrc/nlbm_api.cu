@@ -320,6 +320,30 @@ cudaError_t launch_step(const nlbm_sim *s, const StepParams &kp)
     }
 }
 
+// A simulation in the workspace ws laid out as L (ws nullptr: without state).
+nlbm_status make_sim(const nlbm_params *p, const StepParams &kp, char *ws, const Layout &L, void *cuda_stream,
+                     nlbm_sim **out)
+{
+    nlbm_sim *s = new (std::nothrow) nlbm_sim();
+    if (!s) { set_err(g_err, "host allocation failed"); return NLBM_ENOMEM; }
+    s->kp = kp;
+    s->N = p->n_phases;
+    s->ns = p->n_phases - 1;
+    s->model = p->model;
+    s->storage = p->storage;
+    s->plane = (size_t)p->nx * p->ny;
+    s->stream = (cudaStream_t)cuda_stream;
+    s->ws = ws;
+    s->L = L;
+    s->cur = 0;
+    s->steps = 0;
+    s->launches = 0;
+    s->err[0] = 0;
+    default_tile(s);
+    *out = s;
+    return NLBM_OK;
+}
+
 }  // namespace
 
 extern "C" {
@@ -341,32 +365,14 @@ nlbm_status nlbm_create(const nlbm_params *p, void *dev_workspace, size_t worksp
     StepParams kp;
     nlbm_status st = validate(p, &kp, g_err);
     if (st != NLBM_OK) return st;
-    const int ns = p->n_phases - 1;
-    const Layout L = make_layout(ns, (size_t)p->nx * p->ny, is_half(p->storage));
+    const Layout L = make_layout(p->n_phases - 1, (size_t)p->nx * p->ny, is_half(p->storage));
     if (!dev_workspace) { set_err(g_err, "workspace is NULL"); return NLBM_EINVAL; }
     if (((uintptr_t)dev_workspace & 255) != 0) { set_err(g_err, "workspace must be 256-byte aligned"); return NLBM_EINVAL; }
     if (workspace_bytes < L.total) {
         set_err(g_err, "workspace of %zu bytes is smaller than the %zu needed", workspace_bytes, L.total);
         return NLBM_ENOMEM;
     }
-    nlbm_sim *s = new (std::nothrow) nlbm_sim();
-    if (!s) { set_err(g_err, "host allocation failed"); return NLBM_ENOMEM; }
-    s->kp = kp;
-    s->N = p->n_phases;
-    s->ns = ns;
-    s->model = p->model;
-    s->storage = p->storage;
-    s->plane = (size_t)p->nx * p->ny;
-    s->stream = (cudaStream_t)cuda_stream;
-    s->ws = (char *)dev_workspace;
-    s->L = L;
-    s->cur = 0;
-    s->steps = 0;
-    s->launches = 0;
-    s->err[0] = 0;
-    default_tile(s);
-    *out = s;
-    return NLBM_OK;
+    return make_sim(p, kp, (char *)dev_workspace, L, cuda_stream, out);
 }
 
 nlbm_status nlbm_set_phi(nlbm_sim *s, const float *dev_phi)
@@ -1180,12 +1186,12 @@ const char *nlbm_batch_last_error(const nlbm_batch *b) { return b ? b->err : g_e
 // ------------------------------------------------------------------- adjoint
 
 struct nlbm_adjoint {
-    nlbm_sim *sim;             // forward simulation (its own workspace slice)
+    nlbm_sim *sim;             // parameters, tile and launch count of the steps (no state of its own)
     int ns, N, nsteps, every, nckpt;
     size_t plane, state_floats;
     cudaStream_t stream;
     char *ws;
-    size_t ws_bytes;
+    size_t ws_bytes, sums_bytes;
     float *ckpt;               // [nckpt][state]
     float *seg;                // [every + 1][state]
     float *tapes;              // [every][tape] the rebuilt segment's tapes
@@ -1214,21 +1220,20 @@ constexpr int kUnswept = 3;   // see nlbm_adjoint_forward()
 // m_phi [2] planes (FP32 storage).
 size_t adj_state_floats(int ns, size_t plane) { return plane * ((size_t)ns * 9 + 8 + 2 + ns + 2); }
 
-// Offsets of the per-node arrays of the tape, the two seed sets and the
-// intermediates, in floats per plane.
+// Planes of a step's tape in a sweep, of one seed set and of the
+// intermediates, and values of the parameter gradient (the tensions, M).
 struct AdjCounts {
-    int tape, seedset, inter, contrib;
+    int tape, seedset, inter, params;
 };
 
 AdjCounts adj_counts(int ns)
 {
-    const int np = (ns + 1) * ns / 2;
-    // tape, one seed set, intermediates, per-node gradient sums (FP64: 2 floats each)
-    return AdjCounts{8 * ns + 13, 10 * ns + 12, 9 * ns + 12, 2 * (np + 1)};
+    return AdjCounts{8 * ns + 12, 10 * ns + 12, 9 * ns + 12, (ns + 1) * ns / 2 + 1};
 }
 
 struct AdjLayout {
-    size_t sim, ckpt, seg, tapes, fields, partials, acc, total;
+    size_t ckpt, seg, tapes, fields, sums, partials, acc, total;
+    size_t sums_bytes;   // FP64 sums of the parameter gradient, one a block of the reverse passes
 };
 
 nlbm_status adj_layout(const nlbm_params *p, int nsteps, int every, AdjLayout *L, char *err)
@@ -1252,17 +1257,18 @@ nlbm_status adj_layout(const nlbm_params *p, int nsteps, int every, AdjLayout *L
         off = align256(off + bytes);
         return o;
     };
-    L->sim = take(make_layout(ns, plane, false).total);
     L->ckpt = take(sizeof(float) * adj_state_floats(ns, plane) * nckpt);
     // a segment's states and one spare (the output of its last step), and
     // the tape of each of its steps
     const size_t seglen = (size_t)(every < nsteps ? every : nsteps);
     L->seg = take(sizeof(float) * adj_state_floats(ns, plane) * (seglen + 1));
     L->tapes = take(sizeof(float) * plane * (size_t)c.tape * seglen);
-    // the FP64 per-node sums come first (8-byte alignment)
-    L->fields = take(sizeof(float) * plane * (size_t)(c.contrib + c.tape + 2 * c.seedset + c.inter + 2 * ns + 1));
-    L->partials = take(sizeof(double) * kAdjRedBlocks * c.contrib);
-    L->acc = take(sizeof(double) * c.contrib);
+    // (a single reverse step's tape has one plane more, w)
+    L->fields = take(sizeof(float) * plane * (size_t)(c.tape + 1 + 2 * c.seedset + c.inter + 2 * ns + 1));
+    L->sums_bytes = sizeof(double) * c.params * (size_t)adj_sum_blocks(p->nx, p->ny);
+    L->sums = take(L->sums_bytes);
+    L->partials = take(sizeof(double) * kAdjRedBlocks * c.params);
+    L->acc = take(sizeof(double) * c.params);
     L->total = off;
     return NLBM_OK;
 }
@@ -1367,7 +1373,7 @@ AdjFields adj_fields(const nlbm_adjoint *a, float *so, float *si)
     return A;
 }
 
-// Tape k of the rebuilt segment (the field order of launch_step_tape_{a,b}_f32).
+// Tape k of the segment (the field order of launch_step_tape_{a,b}_f32).
 AdjTape adj_tape(const nlbm_adjoint *a, int k)
 {
     const size_t pl = a->plane;
@@ -1381,8 +1387,8 @@ AdjTape adj_tape(const nlbm_adjoint *a, int k)
     T.lap = b + pl * (5 * ns + 8);
     T.R = b + pl * (6 * ns + 8);
     T.mphi = b + pl * (8 * ns + 8);
-    T.w = b + pl * (8 * ns + 10);
-    T.F = b + pl * (8 * ns + 11);
+    T.w = nullptr;
+    T.F = b + pl * (8 * ns + 10);
     return T;
 }
 
@@ -1401,7 +1407,7 @@ int64_t adj_sweep_launches(const nlbm_adjoint *a, bool rebuild_last)
 cudaError_t adj_backward_body(nlbm_adjoint *a, bool rebuild_last)
 {
     const size_t pl = a->plane, pb = sizeof(float) * pl;
-    const int ns = a->ns, np = (ns + 1) * ns / 2, blocks = adj_sum_blocks(a->sim->kp);
+    const int ns = a->ns, np = (ns + 1) * ns / 2, blocks = adj_sum_blocks(a->sim->kp.nx, a->sim->kp.ny);
     cudaError_t e;
     // No step follows the last: what its first pass gathers (the adjoints of
     // j and of the pulled g in the seed set, of phi in lphi_tot) is 0, and so
@@ -1409,7 +1415,7 @@ cudaError_t adj_backward_body(nlbm_adjoint *a, bool rebuild_last)
     if ((e = cudaMemsetAsync(a->seed[0], 0, pb * (2 * ns + 8), a->stream)) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(a->seed[0] + pl * (10 * ns + 8), 0, pb * 4, a->stream)) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(a->A.lphi_tot, 0, pb * ns, a->stream)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(a->A.gacc, 0, sizeof(double) * (np + 1) * blocks, a->stream)) != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(a->A.gacc, 0, a->sums_bytes, a->stream)) != cudaSuccess) return e;
     if ((e = launch_fold_seed(ns, a->seed_buf, (unsigned)pl, a->seed[0] + pl * (9 * ns + 8), a->stream)) != cudaSuccess)
         return e;
     int cur = 0;
@@ -1470,8 +1476,9 @@ nlbm_status nlbm_adjoint_create(const nlbm_params *p, int32_t nsteps, int32_t ch
     nlbm_adjoint *a = new (std::nothrow) nlbm_adjoint();
     if (!a) { set_err(g_err, "host allocation failed"); return NLBM_ENOMEM; }
     char *ws = (char *)dev_workspace;
-    st = nlbm_create(p, ws + L.sim, make_layout(p->n_phases - 1, (size_t)p->nx * p->ny, false).total, cuda_stream,
-                     &a->sim);
+    StepParams kp;
+    st = validate(p, &kp, g_err);
+    if (st == NLBM_OK) st = make_sim(p, kp, nullptr, Layout{}, cuda_stream, &a->sim);
     if (st != NLBM_OK) {
         delete a;
         return st;
@@ -1498,7 +1505,6 @@ nlbm_status nlbm_adjoint_create(const nlbm_params *p, int32_t nsteps, int32_t ch
         return q;
     };
     const int ns = a->ns;
-    a->A.gacc = (double *)take(c.contrib);
     a->T.phi = take(ns);
     a->T.j = take(2 * ns);
     a->T.g = take(8);
@@ -1521,6 +1527,8 @@ nlbm_status nlbm_adjoint_create(const nlbm_params *p, int32_t nsteps, int32_t ch
     a->A.lphi_tot = take(ns);
     a->seed_buf = take(ns + 1);
     a->grad_buf = take(ns);
+    a->A.gacc = (double *)(ws + L.sums);
+    a->sums_bytes = L.sums_bytes;
     a->partials = (double *)(ws + L.partials);
     a->acc = (double *)(ws + L.acc);
     a->taped = -1;
@@ -1551,7 +1559,7 @@ nlbm_status nlbm_adjoint_forward(nlbm_adjoint *a, const float *dev_phi0, float *
     kp.uout = kp.gout + pl * 8;
     kp.uin = kp.uout;             // one velocity buffer in a record
     kp.phi = kp.uout + pl * 2;
-    kp.pout = s->P(0);
+    kp.pout = a->A.lF;            // the initial pressure is no part of it: into a plane of the sweep's
     const float *src;
     cudaError_t e = initial_fields(dev_phi0, kp.phi, sizeof(float) * pl * ns, a->ws, a->ws_bytes, a->stream, &src);
     if (e != cudaSuccess) return adj_fail(a, e, "copy of the initial phase fields");
@@ -1650,11 +1658,11 @@ nlbm_status nlbm_adjoint_reverse_step(nlbm_adjoint *a, const float *dev_state, c
     const AdjCounts c = adj_counts(ns);
     cudaError_t e;
     if ((e = cudaMemcpyAsync(a->seed[0], dev_seed_out, pb * c.seedset, cudaMemcpyDeviceToDevice, a->stream)) != cudaSuccess ||
-        (e = cudaMemsetAsync(a->A.gacc, 0, pb * c.contrib, a->stream)) != cudaSuccess)
+        (e = cudaMemsetAsync(a->A.gacc, 0, a->sums_bytes, a->stream)) != cudaSuccess)
         return adj_fail(a, e, "seed");
     const StepParams kp = adj_params_from_state(a, dev_state);
     if ((e = launch_reverse_step(ns, kp, a->T, adj_fields(a, a->seed[0], a->seed[1]), false, a->stream)) != cudaSuccess ||
-        (e = launch_grad_reduce(a->A.gacc, np + 1, (unsigned)adj_sum_blocks(kp), a->partials, a->acc, a->stream)) != cudaSuccess)
+        (e = launch_grad_reduce(a->A.gacc, np + 1, (unsigned)adj_sum_blocks(kp.nx, kp.ny), a->partials, a->acc, a->stream)) != cudaSuccess)
         return adj_fail(a, e, "reverse step");
     a->sim->launches += 8;
     double acc[kMaxPhases * kMaxPhases + 1];

@@ -141,9 +141,9 @@ cudaError_t step_form_a_f32(int ns, const StepParams &p, int tx, StepForm *form,
 cudaError_t step_form_b_f32(int ns, const StepParams &p, int tx, StepForm *form, int *wave_rows);
 
 // The FP32 step (128-thread blocks) that also writes the step's
-// intermediate fields for the adjoint to p.tape, 8 (N-1) + 13 planes in the
-// order of AdjTape: phi [N-1], j [2(N-1)], pulled g [8], grad phi [2(N-1)],
-// lap phi [N-1], R [2(N-1)], m_phi [2], w [1], F [2]; Model A in
+// intermediate fields for the adjoint to p.tape, 8 (N-1) + 12 planes: phi
+// [N-1], j [2(N-1)], pulled g [8], grad phi [2(N-1)], lap phi [N-1], R
+// [2(N-1)], m_phi [2], F [2] (of AdjTape, all that a sweep reads); Model A in
 // step_a_f32_tape.cu, Model B in step_b_f32_tape.cu.
 cudaError_t launch_step_tape_a_f32(int ns, const StepParams &p, cudaStream_t st);
 cudaError_t launch_step_tape_b_f32(int ns, const StepParams &p, cudaStream_t st);

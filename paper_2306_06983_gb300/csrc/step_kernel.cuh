@@ -1049,7 +1049,7 @@ __device__ __forceinline__ void complete_node(const StepParams &P, const unsigne
     if (P.pout) P.pout[node] = Pr;
     if constexpr (TAPE) {
         // the intermediate fields of this step at this node, for the
-        // adjoint: phi, j, pulled g, grad phi, lap phi, R, m_phi, w, F
+        // adjoint: phi, j, pulled g, grad phi, lap phi, R, m_phi, F
         float *tp = P.tape + node;
 #pragma unroll
         for (int p = 0; p < NS; ++p) {
@@ -1066,9 +1066,8 @@ __device__ __forceinline__ void complete_node(const StepParams &P, const unsigne
         for (int i = 1; i < 9; ++i) tp[(size_t)(3 * NS + i - 1) * pl] = g[i];
         tp[(size_t)(8 * NS + 8) * pl] = mphx;
         tp[(size_t)(8 * NS + 9) * pl] = mphy;
-        tp[(size_t)(8 * NS + 10) * pl] = w0[0];
-        tp[(size_t)(8 * NS + 11) * pl] = Fx;
-        tp[(size_t)(8 * NS + 12) * pl] = Fy;
+        tp[(size_t)(8 * NS + 10) * pl] = Fx;
+        tp[(size_t)(8 * NS + 11) * pl] = Fy;
     }
 }
 
