@@ -717,16 +717,28 @@ def pair_list(N: int):
     return [(p, q) for p in range(N) for q in range(p + 1, N)]
 
 
-def _final_phi(params: dict, phi0, nsteps: int):
-    """phi(T) [N, ny, nx] of a plain run on phi0's device."""
+def _final_phi(params: dict, phi0, nsteps: int, every: int):
+    """phi(T) [N, ny, nx] of a plain run, without checkpoints and tapes, on
+    phi0's device, after the checks of a differentiable one (the parameters
+    are packed once for all)."""
     import torch
-    sim = Simulation(params, device=phi0.device)
-    t = phi0.to(device=sim.device, dtype=torch.float32).contiguous()
-    out = torch.empty((sim.N, sim.ny, sim.nx), dtype=torch.float32, device=sim.device)
-    nlbm_set_phi(sim.h, t.data_ptr())
-    sim.step(nsteps)
-    nlbm_get_moments(sim.h, ctypes.c_void_p(out.data_ptr()))
-    sim.close()
+    lib, device = load_library(), phi0.device
+    stream = torch.cuda.current_stream(device).cuda_stream
+    s, keep = make_params(params)
+    n, h = ctypes.c_size_t(0), ctypes.c_void_p()
+    _check_adj(lib.nlbm_adjoint_workspace_bytes(ctypes.byref(s), nsteps, every, ctypes.byref(n)))
+    _check(lib.nlbm_workspace_bytes(ctypes.byref(s), ctypes.byref(n)))
+    workspace = torch.empty(n.value + 256, dtype=torch.uint8, device=device)
+    t = phi0.to(dtype=torch.float32).contiguous()
+    out = torch.empty((s.n_phases, s.ny, s.nx), dtype=torch.float32, device=device)
+    _check(lib.nlbm_create(ctypes.byref(s), ctypes.c_void_p((workspace.data_ptr() + 255) // 256 * 256), n.value,
+                           ctypes.c_void_p(stream), ctypes.byref(h)))
+    try:
+        nlbm_set_phi(h, t.data_ptr())
+        nlbm_step(h, nsteps)
+        nlbm_get_moments(h, ctypes.c_void_p(out.data_ptr()))
+    finally:
+        nlbm_destroy(h)
     return out
 
 
@@ -747,10 +759,7 @@ def _make_function():
                 sig[p, q] = sig[q, p] = v
             q = dict(params, sigma=sig.tolist(), mobility=float(mobility.detach().cpu()))
             if not sweep:
-                # no gradient will be asked for: a plain run, without
-                # checkpoints and tapes, of what a differentiable one takes
-                nlbm_adjoint_workspace_bytes(q, nsteps, every)
-                return _final_phi(q, phi0.detach(), nsteps)
+                return _final_phi(q, phi0.detach(), nsteps, every)   # no gradient will be asked for
             run = AdjointRun(q, nsteps, every, device=phi0.device)
             out = run.forward(phi0.detach())
             ctx.run = run
