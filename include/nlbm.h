@@ -200,11 +200,13 @@ int64_t nlbm_kernel_launches(const nlbm_sim *s);
 
 /* Tile of the fused step kernel: tx threads per block (64, 128 or 256; one
  * thread per column, each block updating a strip of tx - 4 columns) marching
- * down ty rows (>= 1), or ty = 0 (the default) to let the library choose:
- * patches of 16 or 32 columns and 8 rows where marches would be short, else
- * every strip cut into equal row chunks (at least 2 rows) so that the grid
- * is one wave of resident blocks.  With 16-bit storage the step always runs
- * on patches.  Results do not depend on the tile.  EINVAL outside those
+ * down ty rows (>= 1), or ty = 0 (the default) to let the library choose
+ * what costs least by its measure: patches of 16 or 32 columns and 8 rows
+ * (most small lattices, and all with N = 3), every strip cut into equal row
+ * chunks (at least 2 rows) so that the grid is one wave of resident blocks,
+ * or, for large lattices with N = 5 or 6, strips of 60 columns marched down 20
+ * rows; of these only the one-wave march depends on tx.  With 16-bit storage
+ * the step always runs on patches, whatever the tile.  Results do not depend on the tile.  EINVAL outside those
  * values.  Takes effect on the next nlbm_step(). */
 nlbm_status nlbm_set_tile(nlbm_sim *s, int32_t tx, int32_t ty);
 nlbm_status nlbm_get_tile(const nlbm_sim *s, int32_t *tx, int32_t *ty);

@@ -21,7 +21,7 @@
 // rev2 and rev3 (rev_source_kernel).  Against one launch per pass, per-node
 // FP64 gradient sums and the same taping rebuild: 1024^2 N = 3 (Model B)
 // backward 249 -> 211 us a step, 256^2 24.1 -> 20.4.  The collision pass
-// moves 4.0 TB/s of DRAM traffic at 24 warps an SM (80 registers) and 39 %
+// moves 4.5 TB/s of DRAM traffic at 21 warps an SM (80 registers) and 44 %
 // issue; more loads in flight (its inputs staged by cp.async) did not change
 // its time, nor did precomputed neighbour offsets.
 // The adjoint of the step's inputs is the seed of the previous step.  The

@@ -790,7 +790,9 @@ struct OwnRing {
 
 // a b + c d with the first product fused.  Left to the compiler, which of the
 // two is fused depends on the code around the sum, and the row march and the
-// patch kernel have to give the same bits.
+// patch kernel have to give the same bits.  Written out where the compiler had
+// chosen differently in the two; elsewhere it chooses alike (compared bit for
+// bit in tests for both models at every phase count and form of the step).
 __device__ __forceinline__ float two_products(float a, float b, float c, float d)
 {
     return __fmaf_rn(a, b, __fmul_rn(c, d));

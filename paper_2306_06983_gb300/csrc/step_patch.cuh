@@ -1,4 +1,6 @@
-// The fused step on patches, for lattices whose row marches would be short.
+// The fused step on patches: where row marches would be short, where their
+// strips fit the lattice badly, for the phase counts and models that run
+// faster so at any size (use_patches), and for 16-bit storage.
 //
 // step_tile marches a strip of columns down the lattice: every row costs one
 // round trip to memory and two barriers, and each chunk repeats 4 + 2
@@ -281,7 +283,7 @@ template <int NS, int MODEL, int ST, bool TAPE>
 cudaError_t launch_patches(const StepParams &p, cudaStream_t st)
 {
     constexpr int kNarrowMin = NS <= 3 ? 6 : (NS <= 5 ? 5 : 4), kWideMin = NS <= 2 ? 4 : (NS <= 4 ? 3 : 2);
-    constexpr int kFill = 228;   // wide patches from 1.5 per SM on (256^2: equal, 300x150: 8 % slower)
+    constexpr int kFill = 152 * 3 / 2;   // wide patches from 1.5 per SM on (256^2: equal, 300x150: 8 % slower)
     if constexpr (wide_patches<NS, MODEL, ST>()) {
         if ((long long)((p.nx + 31) / 32) * ((p.ny + 7) / 8) >= kFill)
             return launch_patch_variant<NS, MODEL, ST, 32, 8, kWideMin, TAPE>(p, st);
