@@ -206,8 +206,9 @@ int64_t nlbm_kernel_launches(const nlbm_sim *s);
  * chunks (at least 2 rows) so that the grid is one wave of resident blocks,
  * or, for large lattices with N = 5 or 6, strips of 60 columns marched down 20
  * rows; of these only the one-wave march depends on tx.  With 16-bit storage
- * the step always runs on patches, whatever the tile.  Results do not depend on the tile.  EINVAL outside those
- * values.  Takes effect on the next nlbm_step(). */
+ * the step always runs on patches, whatever the tile.  Results do not depend
+ * on the tile.  EINVAL outside those values.  Takes effect on the next
+ * nlbm_step(). */
 nlbm_status nlbm_set_tile(nlbm_sim *s, int32_t tx, int32_t ty);
 nlbm_status nlbm_get_tile(const nlbm_sim *s, int32_t *tx, int32_t *ty);
 
