@@ -89,3 +89,42 @@ def test_ensemble_and_gradient_run(where):
         b.close()
         run.close()
     assert all(torch.equal(x, y) for x, y in zip(*out))
+
+
+def test_captured_into_a_graph():
+    """set_phi and steps under stream capture: a replay takes the fields that
+    the array holds then."""
+    import torch
+    from paper_2306_06983_gb300.nlbm import Simulation
+    p, phi0 = W.random_smooth(NX, NY, N, seed=6, model="B", n_disks=3)
+    phi0 = torch.from_numpy(phi0.astype(np.float32)).cuda()
+    flipped = phi0.flip(2).contiguous()
+    plain = Simulation(p)
+    want = []
+    for f in (phi0, flipped):
+        plain.set_phi(f)
+        plain.step(4)
+        want.append(plain.moments())
+    buf = phi0.clone()
+    stream = torch.cuda.Stream()
+    stream.wait_stream(torch.cuda.current_stream())
+    sim = Simulation(p, stream=stream)
+    with torch.cuda.stream(stream):
+        sim.set_phi(buf)   # loads the kernels
+        sim.step(4)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        sim.set_phi(buf)
+        sim.step(4)
+    for f, w in zip((phi0, flipped), want):
+        buf.copy_(f)
+        torch.cuda.synchronize()
+        graph.replay()
+        torch.cuda.synchronize()
+        with torch.cuda.stream(stream):
+            got = sim.moments()
+        torch.cuda.synchronize()
+        assert all(torch.equal(a, b) for a, b in zip(got, w))
+    sim.close()
+    plain.close()
