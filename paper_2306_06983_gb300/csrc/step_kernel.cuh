@@ -1472,7 +1472,7 @@ StepForm auto_form(const StepParams &p, int T, int slots)
             nodes = narrow;
         }
     }
-    return use_patches<NS, MODEL>(p, nodes, windows) ? StepForm::Patches : form;
+    return use_patches<NS, MODEL, TAPE>(p, nodes, windows) ? StepForm::Patches : form;
 }
 
 template <int NS, int MODEL, int T, bool TAPE = false>

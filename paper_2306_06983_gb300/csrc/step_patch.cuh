@@ -301,9 +301,25 @@ cudaError_t launch_patches(const StepParams &p, cudaStream_t st)
 // 114 / 91; 1472^2 N = 6 222 / 243).  1: patches at every size (2048^2 N = 3 200 /
 // 192); so it is for most lattices without row windows (1279^2 N = 6 234 / 203,
 // 2045^2 N = 8 761 / 700).
-template <int NS, int MODEL>
+//
+// The taping step writes another 8 NS + 12 planes, which patches write best
+// where their rows of 32 columns start on a 32-byte sector (nx a multiple of
+// 8): there they are ahead at almost any size, elsewhere marches are on large
+// lattices (us a step of a taped forward of 8 steps, march / patches, Model B:
+// 1024^2 N = 3 86 / 78, N = 5 154 / 127, 1472^2 N = 4 250 / 200; 1100^2 N = 6 189 /
+// 223, 868 x 1024 N = 2 53 / 58; 1279^2 N = 3 152 / 164, N = 5 249 / 306, but N = 7
+// 408 / 348).
+template <int NS, int MODEL, bool TAPE>
 inline bool use_patches(const StepParams &p, double march_nodes, bool windows)
 {
+    if constexpr (TAPE) {
+        // nx a multiple of 8; of 4; no row windows
+        constexpr bool A = MODEL == 0;
+        constexpr double kTape[3][7] = {{1., 1., 1., 1., A ? 1. : .89, 1., A ? .965 : .92},
+                                        {.85, .85, 1., A ? 1. : .85, .85, .90, .85},
+                                        {.82, .75, .83, .75, .75, 1., 1.}};
+        return kTape[windows ? (p.nx % 8 != 0) : 2][NS - 1] * march_nodes >= (double)p.nx * p.ny;
+    }
     constexpr double kGain[2][7] = {{.865, 1., .905, .965, .93, .88, .9725}, {.865, 1., .905, .895, .92, .88, .82}};
     const double gain = windows ? kGain[MODEL][NS - 1] : NS == 1 ? .835 : NS == 4 && MODEL == 1 ? .90 : 1.;
     return gain * march_nodes >= (double)p.nx * p.ny;
